@@ -145,6 +145,48 @@ constexpr MtInverse make_mt_inverse() {
 }
 constexpr MtInverse kMtInv = make_mt_inverse();
 
+// ---- arithmetic ------------------------------------------------------------------------
+// The collision is written in single-rounding operations (no contraction left to the
+// compiler), so every kernel that runs it -- one cell per thread, two cells per thread on
+// the paired FP32 instructions, staged -- produces the same bits.  pf2 is a pair of cells
+// in one 64-bit register pair: one FFMA2 / FADD2 / FMUL2 does both cells' operation in one
+// issue slot (the same FP32 lane rate as two scalar instructions, half the issue slots).
+using pf2 = float2;
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float neg_(float a) { return -a; }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double neg_(double a) { return -a; }
+__device__ __forceinline__ pf2 fma_(pf2 a, pf2 b, pf2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ pf2 mul_(pf2 a, pf2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ pf2 add_(pf2 a, pf2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ pf2 sub_(pf2 a, pf2 b) { return fma_(b, make_float2(-1.f, -1.f), a); }   // same rounding
+__device__ __forceinline__ pf2 neg_(pf2 a) { return make_float2(-a.x, -a.y); }
+
+// The scalar type of R and a constant of type R.
+template <class R> struct scalar_of { using type = R; };
+template <> struct scalar_of<pf2> { using type = float; };
+template <class R> __device__ __forceinline__ R lit(typename scalar_of<R>::type c) {
+    if constexpr (std::is_same<R, pf2>::value) return make_float2(c, c);
+    else return c;
+}
+
+// 1 / x.  FP32: the hardware's approximate reciprocal and one Newton-Raphson iteration
+// r + r (1 - x r), which leaves it within one unit in the last place over the normal range
+// (x is a density, near 1) in three instructions and without the branch of the division.
+__device__ __forceinline__ float recip_(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_rn(r, __fmaf_rn(-x, r, 1.f), r);
+}
+__device__ __forceinline__ double recip_(double x) { return 1.0 / x; }
+__device__ __forceinline__ pf2 recip_(pf2 x) { return make_float2(recip_(x.x), recip_(x.y)); }
+
 // ---- storage ------------------------------------------------------------------------
 // ld / st convert between the stored value and f - w; ldr / str move the stored value
 // unscaled (the step kernels of the scaled half format work in units of 2^-s, see collide).
@@ -227,11 +269,18 @@ struct Member {
     const void *ztab;          // trigger: [2][nz] cos, sin of kz 2 pi z / L, compute type
     const void *dtab;          // Bouzidi walls: [ny][nx][9][3] coefficients A, B, C of the link
                                // (cx, cy) at index nbit(cx, cy), compute type
+    const uint32_t *pairinfo;  // compact: [Ps / 2] per pair of stored positions (see PAIR_*)
+    const void *ftabc;         // trigger, compact: [3][Ps] column factors by stored position
     const int4 *sg[2];         // compact: row groups of the two staged launch shapes (2 int4
                                // per group, see lbm_staged.cuh), nsg[k] groups (0: shape
                                // not available for this member)
     int32_t nsg[2];
 };
+
+// An entry of pairinfo: whether the first and the second position are fluid cells, whether
+// one of them has a wall link, and the dense column y nx + x of the first.
+constexpr uint32_t PAIR_A = 1, PAIR_B = 2, PAIR_WALL = 4;
+constexpr int PAIR_SHIFT = 3;
 
 // Unsigned division by a fixed divisor d >= 1 for n < 2^31 (Granlund-Montgomery with
 // a 31-bit dividend): l = ceil(log2 d), mul = ceil(2^(31+l) / d) < 2^32, and
@@ -273,6 +322,8 @@ struct StepArgs {
     int32_t tidx;
     void *moments;            // adjoint recompute: [9][cells] rho, u, s4..s8 of member 0
     int32_t collision;        // collision model (MODEL_* bits), the same for every member
+    uint32_t zero;            // 0 (see store_pops)
+    int32_t pairs;            // an even step on pairs of cells (lbm_pair.cuh)
     int32_t stage_cap;        // staged shapes: storage elements per direction segment
     int32_t sg_sel;           // staged shapes: which row-group table (0 or 1)
     int32_t *err;             // device status word (bounded waits that expired), or NULL
@@ -434,7 +485,7 @@ __device__ __forceinline__ void bouzidi_load_fix(const Member &d, const CellPos 
         if constexpr (cx_of(j) != 0 || cy_of(j) != 0) {
             if (!dst_is_fluid<j>(p)) {
                 BLink<R> b = bouzidi_link<R, j>(d, p);
-                v[opp_of(j)] += b.C * v[j];
+                v[opp_of(j)] = fma_(b.C, v[j], v[opp_of(j)]);
             }
         }
     });
@@ -492,9 +543,11 @@ __device__ __forceinline__ void store_pops(const StepArgs &a, const Member &d, c
     using S = Storage<P>;
     using T = typename S::T;
     using R = typename S::R;
-    T *base = static_cast<T *>(a.pops) + d.off;
-    const uint32_t st = (uint32_t)a.stride;
-    const uint32_t lc = (uint32_t)p.lc;
+    // a slot is written where it was read: the zero keeps the compiler from carrying the 27
+    // addresses through the collision in registers
+    T *base = static_cast<T *>(a.pops) + d.off + a.zero;
+    const uint32_t st = (uint32_t)a.stride + a.zero;
+    const uint32_t lc = (uint32_t)p.lc + a.zero;
     const R sc = (R)a.f16_scale;
     if constexpr (WALL == LBM_BOUZIDI) {
         // the value reflected into slot Jbar becomes A f*_J + B f*_Jbar
@@ -506,7 +559,7 @@ __device__ __forceinline__ void store_pops(const StepArgs &a, const Member &d, c
                 if constexpr (cx_of(j) != 0 || cy_of(j) != 0) {
                     if (!dst_is_fluid<j>(p)) {
                         BLink<R> b = bouzidi_link<R, j>(d, p);
-                        out[j] = b.A * v[j] + b.B * v[opp_of(j)];
+                        out[j] = fma_(b.A, v[j], mul_(b.B, v[opp_of(j)]));
                     }
                 }
             });
@@ -519,7 +572,7 @@ __device__ __forceinline__ void store_pops(const StepArgs &a, const Member &d, c
         if constexpr (PAR == 0) {
             st_pop<P, RAW>(base + (ib * st + lc), v[i], sc);
         } else {
-            const uint32_t push = i * st + (uint32_t)(p.lc + nb_offset<i>(p));
+            const uint32_t push = i * st + (lc + (uint32_t)nb_offset<i>(p));
             if constexpr (WALL == LBM_FULLWAY || (cx_of(i) == 0 && cy_of(i) == 0)) {
                 st_pop<P, RAW>(base + push, v[i], sc);
             } else {
@@ -563,10 +616,10 @@ __device__ __forceinline__ void acceleration(const Member &d, const CellPos &p, 
         const R *ft = static_cast<const R *>(d.ftab);
         const R *zt = static_cast<const R *>(d.ztab);
         const int32_t col = p.y * d.nx + p.x, ncol = d.nx * d.ny;
-        const R sc = st * zt[p.z], ss = st * zt[d.nz + p.z];
-        gx += sc * ft[col];
-        gy += sc * ft[ncol + col];
-        gz += ss * ft[2 * ncol + col];
+        const R sc = mul_(st, zt[p.z]), ss = mul_(st, zt[d.nz + p.z]);
+        gx = fma_(sc, ft[col], gx);
+        gy = fma_(sc, ft[ncol + col], gy);
+        gz = fma_(ss, ft[2 * ncol + col], gz);
     }
 }
 
@@ -606,7 +659,7 @@ __device__ __forceinline__ void trigger_column(const Member &d, int x, int y, do
 
 // ---- collision ------------------------------------------------------------------------------
 template <class R>
-struct Macro { R drho, rho, ux, uy, uz; };
+struct Macro { R rho, ux, uy, uz; };
 
 // The moments a collision needs, from v = f - w: drho = sum f - 1, j = sum c f and the raw
 // second moments m4..m8 of Eq. (Mmatrix) (xy, xz, yz, x^2 - y^2, x^2 - z^2; the weights
@@ -622,50 +675,76 @@ __device__ __forceinline__ MomentSums<R> moment_sums(const R (&v)[Q]) {
     sfor<0, 9>([&](auto kc) {                       // column (cx, cy) = (a - 1, b - 1)
         constexpr int k = decltype(kc)::value, a = k % 3, b = k / 3;
         constexpr int ip = dir_of(a - 1, b - 1, 1), im = dir_of(a - 1, b - 1, -1), i0 = dir_of(a - 1, b - 1, 0);
-        P[a][b] = v[ip] + v[im];
-        S[a][b] = P[a][b] + v[i0];
-        D[a][b] = v[ip] - v[im];
+        P[a][b] = add_(v[ip], v[im]);
+        S[a][b] = add_(P[a][b], v[i0]);
+        D[a][b] = sub_(v[ip], v[im]);
     });
     MomentSums<R> m;
-    R Sa[3], Sb[3], Da[3];
+    R Sa[3], Da[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        Sa[k] = S[k][0] + S[k][1] + S[k][2];     // column sums at cx = k - 1
-        Sb[k] = S[0][k] + S[1][k] + S[2][k];     // at cy = k - 1
-        Da[k] = D[k][0] + D[k][1] + D[k][2];
+        Sa[k] = add_(add_(S[k][0], S[k][1]), S[k][2]);     // column sums at cx = k - 1
+        Da[k] = add_(add_(D[k][0], D[k][1]), D[k][2]);
     }
-    m.drho = Sa[0] + Sa[1] + Sa[2];
-    m.jx = Sa[2] - Sa[0];
-    m.jy = Sb[2] - Sb[0];
-    m.jz = Da[0] + Da[1] + Da[2];
-    m.m4 = (S[2][2] - S[2][0]) - (S[0][2] - S[0][0]);
-    m.m5 = Da[2] - Da[0];
-    m.m6 = (D[0][2] - D[0][0]) + (D[1][2] - D[1][0]) + (D[2][2] - D[2][0]);
-    m.m7 = (S[0][1] + S[2][1]) - (S[1][0] + S[1][2]);
+    const R Sb0 = add_(add_(S[0][0], S[1][0]), S[2][0]);   // at cy = -1, +1
+    const R Sb2 = add_(add_(S[0][2], S[1][2]), S[2][2]);
+    m.drho = add_(add_(Sa[0], Sa[1]), Sa[2]);
+    m.jx = sub_(Sa[2], Sa[0]);
+    m.jy = sub_(Sb2, Sb0);
+    m.jz = add_(add_(Da[0], Da[1]), Da[2]);
+    m.m4 = sub_(sub_(S[2][2], S[2][0]), sub_(S[0][2], S[0][0]));
+    m.m5 = sub_(Da[2], Da[0]);
+    m.m6 = sub_(add_(add_(D[0][2], D[1][2]), D[2][2]), add_(add_(D[0][0], D[1][0]), D[2][0]));
+    m.m7 = sub_(add_(S[0][1], S[2][1]), add_(S[1][0], S[1][2]));
     // x^2 - z^2: +1 on the cz = 0 populations of the cx != 0 columns, -1 on the cz != 0
     // populations of the cx = 0 columns
     constexpr int a0 = dir_of(-1, -1, 0), a1 = dir_of(-1, 0, 0), a2 = dir_of(-1, 1, 0);
     constexpr int b0 = dir_of(1, -1, 0), b1 = dir_of(1, 0, 0), b2 = dir_of(1, 1, 0);
-    const R f0x = ((v[a0] + v[b0]) + (v[a1] + v[b1])) + (v[a2] + v[b2]);
-    m.m8 = f0x - (P[1][0] + P[1][1] + P[1][2]);
+    const R f0x = add_(add_(add_(v[a0], v[b0]), add_(v[a1], v[b1])), add_(v[a2], v[b2]));
+    m.m8 = sub_(f0x, add_(add_(P[1][0], P[1][1]), P[1][2]));
     return m;
 }
 
-template <class R>
-__device__ __forceinline__ Macro<R> macro_from_sums(const MomentSums<R> &s, R gx, R gy, R gz) {
+// rho and u = sum c f / rho + g / 2 from the sums (bare momentum j, hg = g / 2).  SCALED: the
+// sums are in units of inv = 2^-s (the scaled half format; powers of two, exact).
+// u = j + (g / 2 - j (rho - 1) / rho): the bracket is small, so u is rounded once, where
+// j (1 / rho) + g / 2 also carries the reciprocal's rounding; the rounding of u moves the
+// momentum of all 18 moving populations alike and does not average out over the steps.
+// LEAN takes u = j (1 / rho) + g / 2: FP64, and the 16-bit formats, whose storage rounds
+// 4,000 times coarser.
+template <class R, bool SCALED = false, bool LEAN = false>
+__device__ __forceinline__ Macro<R> macro_from_sums(const MomentSums<R> &s, R hgx, R hgy, R hgz,
+                                                    typename scalar_of<R>::type inv = 1) {
     Macro<R> m;
-    m.drho = s.drho;
-    m.rho = R(1) + s.drho;
-    const R ir = R(1) / m.rho;
-    m.ux = s.jx * ir + R(0.5) * gx;
-    m.uy = s.jy * ir + R(0.5) * gy;
-    m.uz = s.jz * ir + R(0.5) * gz;
+    R jx = s.jx, jy = s.jy, jz = s.jz;
+    if constexpr (LEAN) {
+        if constexpr (SCALED) m.rho = fma_(s.drho, lit<R>(inv), lit<R>(1));
+        else m.rho = add_(s.drho, lit<R>(1));
+        R ir = recip_(m.rho);
+        if constexpr (SCALED) ir = mul_(ir, lit<R>(inv));
+        m.ux = fma_(jx, ir, hgx);
+        m.uy = fma_(jy, ir, hgy);
+        m.uz = fma_(jz, ir, hgz);
+        return m;
+    }
+    if constexpr (SCALED) {
+        m.rho = fma_(s.drho, lit<R>(inv), lit<R>(1));
+        jx = mul_(jx, lit<R>(inv));
+        jy = mul_(jy, lit<R>(inv));
+        jz = mul_(jz, lit<R>(inv));
+    } else {
+        m.rho = add_(s.drho, lit<R>(1));
+    }
+    const R nq = mul_(sub_(lit<R>(1), m.rho), recip_(m.rho));
+    m.ux = add_(jx, fma_(jx, nq, hgx));
+    m.uy = add_(jy, fma_(jy, nq, hgy));
+    m.uz = add_(jz, fma_(jz, nq, hgz));
     return m;
 }
 
 template <class R>
 __device__ __forceinline__ Macro<R> macroscopic(const R (&v)[Q], R gx, R gy, R gz) {
-    return macro_from_sums<R>(moment_sums<R>(v), gx, gy, gz);
+    return macro_from_sums<R, false, sizeof(R) == 8>(moment_sums<R>(v), mul_(lit<R>(0.5f), gx), mul_(lit<R>(0.5f), gy), mul_(lit<R>(0.5f), gz));
 }
 
 // One-axis factors of the product-form equilibrium (see the file header):
@@ -696,6 +775,130 @@ template <int E, class R> __device__ __forceinline__ R cterm(R acc, R x) {
     else return acc;
 }
 
+// The default model's post-collision populations from the moment sums of a cell (R float,
+// double) or of a pair of cells (R pf2): emit(i, f*_i - w_i) for every i, row of columns
+// (c_y) by row.  SCALED (the scaled half format): sums and outputs are in storage
+// units, (f - w) sc with sc = 1 / inv a power of two; the shear moments stay in those units
+// and sc enters the density constants, which is exact.
+//
+//   f*_i - w_i = w_i drho + w_i rho X_i + (shear term), X_i = f^eq / (w rho) - 1 +
+//   (1/2) g . grad_u (f^eq / (w rho)).
+//
+// With the one-axis factors p = psi_hat, d = p - 1, h = (g/2) psi_hat', per in-plane column
+// D = px py - 1 = dx + dy px and G = D + hx py + hy px, X = G + hz (1 + D) + dz (1 + G): the
+// force meets dz only in the last sum, whose rounding differs from column to column (added to
+// dz once for all columns, its rounding adds up over them and the mean flow drifts: the error
+// of u after 100 steps doubles).  The shear moments use the bare momentum j and p = j +
+// rho g / 2: m_k - m_k^eq + R_k / 2 collapses to m4 - j_x u_y + (g_y / 2) p_x and its like.
+// About 290 FP32 operations per cell (330 with rho u u products and separate weights); emitting
+// row by row keeps the live set small.
+// ACT: the outputs are multiplied by act (1, or 0 for the padding half of a pair, which must
+// stay zero) through the four factors they all carry.
+// LEAN (see macro_from_sums): X = G (1 + dz) + hz D + (dz + hz), 15 operations fewer.
+template <class R, bool SCALED, bool ACT, bool LEAN, class Emit>
+__device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R gy, R gz,
+                                                typename scalar_of<R>::type omega, typename scalar_of<R>::type inv,
+                                                typename scalar_of<R>::type sc, R *s_out, Emit &&emit,
+                                                R act = lit<R>(1)) {
+    using S = typename scalar_of<R>::type;
+    const R hgx = mul_(lit<R>(0.5f), gx), hgy = mul_(lit<R>(0.5f), gy), hgz = mul_(lit<R>(0.5f), gz);
+    const Macro<R> mm = macro_from_sums<R, SCALED, LEAN>(ms, hgx, hgy, hgz, inv);
+    const R rho = mm.rho;
+    // non-equilibrium shear moments s4..s8 (p = j + rho g / 2, in the units of the sums)
+    const R rs = SCALED ? mul_(rho, lit<R>(sc)) : rho;
+    const R px_ = fma_(rs, hgx, ms.jx), py_ = fma_(rs, hgy, ms.jy), pz_ = fma_(rs, hgz, ms.jz);
+    const R njx = neg_(ms.jx), njy = neg_(ms.jy);
+    const R s4 = fma_(njx, mm.uy, fma_(hgy, px_, ms.m4));
+    const R s5 = fma_(njx, mm.uz, fma_(hgz, px_, ms.m5));
+    const R s6 = fma_(njy, mm.uz, fma_(hgz, py_, ms.m6));
+    const R tx = fma_(njx, mm.ux, mul_(hgx, px_));            // -rho (u_x^2 - g_x u_x)
+    const R ty = fma_(njy, mm.uy, mul_(hgy, py_));
+    const R tz = fma_(neg_(ms.jz), mm.uz, mul_(hgz, pz_));
+    const R s7 = sub_(add_(ms.m7, tx), ty);
+    const R s8 = sub_(add_(ms.m8, tx), tz);
+    if (s_out) {
+        s_out[0] = s4; s_out[1] = s5; s_out[2] = s6; s_out[3] = s7; s_out[4] = s8;
+    }
+    // (1 - omega) C_k s_k on the populations with the matching velocity products
+    const S om1 = S(1) - omega;
+    R om6 = lit<R>(om1 * S(1.0 / 6.0)), om4 = lit<R>(om1 * S(0.25)), rho_o = rho, drho_o = ms.drho;
+    if constexpr (ACT) {
+        om6 = mul_(om6, act);
+        om4 = mul_(om4, act);
+        rho_o = mul_(rho_o, act);
+        drho_o = mul_(drho_o, act);
+    }
+    const R b7 = mul_(om6, s7), b8 = mul_(om6, s8);
+    const R s12 = fma_(om6, s7, b8), s34 = fma_(lit<R>(-2), b7, b8), s56 = fma_(lit<R>(-2), b8, b7);
+    const R q4 = mul_(om4, s4), q5 = mul_(om4, s5), q6 = mul_(om4, s6);
+    // one-axis factors at c = -1, 0, +1: d, h and p = 1 + d (those of x row by row).  No sum
+    // takes a product that is rounded by itself: the compiler fuses those on pairs and not on
+    // single cells, and the two would differ in the last bit.
+    auto axis = [](auto cc, R u, R hg, R &d, R &h, R &p) {
+        constexpr int c = decltype(cc)::value;
+        const R u2 = mul_(u, u), t = mul_(lit<R>(3), u), h3 = mul_(lit<R>(3), hg), w = mul_(h3, u);
+        if constexpr (c == 1) {
+            d = mul_(lit<R>(-1.5f), u2);
+            h = neg_(w);
+            p = fma_(lit<R>(-1.5f), u2, lit<R>(1));
+        } else {
+            d = fma_(lit<R>(3), u2, c == 0 ? neg_(t) : t);
+            h = fma_(lit<R>(2), w, c == 0 ? neg_(h3) : h3);
+            p = add_(d, lit<R>(1));
+        }
+    };
+    R dy[3], hy[3], py[3], dz[3], hz[3], pz[3], ez[3];
+    sfor<0, 3>([&](auto cc) {
+        constexpr int c = decltype(cc)::value;
+        axis(cc, mm.uy, hgy, dy[c], hy[c], py[c]);
+        axis(cc, mm.uz, hgz, dz[c], hz[c], pz[c]);
+        if constexpr (c == 1) ez[c] = fma_(lit<R>(-1.5f), mul_(mm.uz, mm.uz), hz[c]);
+        else ez[c] = add_(dz[c], hz[c]);
+    });
+    // w rho and w drho (plus the shear term of the population) per weight shell
+    const S f = SCALED ? sc : S(1);
+    const R wr0 = mul_(lit<R>(S(w_of(0)) * f), rho_o), wr1 = mul_(lit<R>(S(w_of(1)) * f), rho_o);
+    const R wr2 = mul_(lit<R>(S(w_of(7)) * f), rho_o), wr3 = mul_(lit<R>(S(w_of(19)) * f), rho_o);
+    const R w1 = lit<R>(S(w_of(1))), w2 = lit<R>(S(w_of(7)));
+    const R wd0 = mul_(lit<R>(S(w_of(0))), drho_o), wd3 = mul_(lit<R>(S(w_of(19))), drho_o);
+    const R c12 = fma_(w1, drho_o, s12), c34 = fma_(w1, drho_o, s34), c56 = fma_(w1, drho_o, s56);
+    const R c4p = fma_(w2, drho_o, q4), c4m = fma_(w2, drho_o, neg_(q4)), c5p = fma_(w2, drho_o, q5);
+    const R c5m = fma_(w2, drho_o, neg_(q5)), c6p = fma_(w2, drho_o, q6), c6m = fma_(w2, drho_o, neg_(q6));
+    sfor<0, 3>([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        R dx, hx, px;
+        axis(ac, mm.ux, hgx, dx, hx, px);
+        sfor<0, 3>([&](auto bc) {
+            constexpr int b = decltype(bc)::value;
+            const R D = fma_(dy[b], px, dx);
+            const R G = fma_(hx, py[b], fma_(hy[b], px, D));
+            const R A = add_(D, lit<R>(1)), H = add_(G, lit<R>(1));
+            sfor<0, 3>([&](auto cc) {
+                constexpr int c = decltype(cc)::value, i = dir_of(a - 1, b - 1, c - 1);
+                R X;
+                if constexpr (LEAN) X = fma_(G, pz[c], fma_(hz[c], D, ez[c]));
+                else X = fma_(dz[c], H, fma_(hz[c], A, G));
+                R wr, wd;
+                if constexpr (i == 0) { wr = wr0; wd = wd0; }
+                else if constexpr (i <= 6) {
+                    wr = wr1;
+                    wd = (i <= 2) ? c12 : ((i <= 4) ? c34 : c56);
+                } else if constexpr (i <= 18) {
+                    wr = wr2;
+                    if constexpr (i == 7 || i == 10) wd = c4p;
+                    else if constexpr (i == 8 || i == 9) wd = c4m;
+                    else if constexpr (i == 11 || i == 14) wd = c5p;
+                    else if constexpr (i == 12 || i == 13) wd = c5m;
+                    else if constexpr (i == 15 || i == 18) wd = c6p;
+                    else wd = c6m;
+                } else { wr = wr3; wd = wd3; }
+                emit(std::integral_constant<int, i>{}, fma_(wr, X, wd));
+            });
+        });
+    });
+    return mm;
+}
+
 // In-place collision of one fluid cell; v holds f - w on entry and f* - w on exit.
 // With s_out, the five non-equilibrium shear moments s_k = m_k - m_k^eq + R_k / 2
 // (k = 4..8) are returned as well (the adjoint stores them).
@@ -705,182 +908,123 @@ template <int E, class R> __device__ __forceinline__ R cterm(R acc, R x) {
 // is the same for both equilibria since they share their second moments and those of F;
 // for the BGK, N = f - f^eq + F/2.  MODEL_RATES takes a general diagonal Lambda:
 // f* = f^eq + F/2 + (M^T)^{-1} (1 - Lambda) M^T n with n = f - f^eq + F/2, whose moments
-// 0..3 vanish (lam1[k - 4] = 1 - lambda_k).
-//
-// SCALED (default model only): v holds (f - w) sc on entry and leaves with (f* - w) sc,
-// sc = 1 / inv a power of two (the half format's scale): the moment sums are taken in
-// those units and multiplied by inv once, and sc enters the output constants, which is
-// exact and saves the per-population scaling of loads and stores.
-template <class R, int MODEL = MODEL_MRT_H6, bool SCALED = false>
+// 0..3 vanish (lam1[k - 4] = 1 - lambda_k).  The default model runs collide_mrt; SCALED
+// (default model only): v is in storage units, see there.
+template <class R, int MODEL = MODEL_MRT_H6, bool SCALED = false, bool LEAN = sizeof(R) == 8>
 __device__ __forceinline__ Macro<R> collide(R (&v)[Q], R gx, R gy, R gz, R omega, R *s_out = nullptr,
                                             const R *lam1 = nullptr, R inv = R(1), R sc = R(1)) {
-    constexpr bool rates = (MODEL & MODEL_RATES) != 0;
-    constexpr bool bgk = !rates && (MODEL & MODEL_BGK) != 0, o2 = (MODEL & MODEL_O2) != 0;
     static_assert(!SCALED || MODEL == MODEL_MRT_H6, "scaled units serve the default model only");
-    MomentSums<R> ms = moment_sums<R>(v);
-    if constexpr (SCALED) {
-        ms.drho *= inv; ms.jx *= inv; ms.jy *= inv; ms.jz *= inv;
-        ms.m4 *= inv; ms.m5 *= inv; ms.m6 *= inv; ms.m7 *= inv; ms.m8 *= inv;
-    }
-    const Macro<R> mm = macro_from_sums<R>(ms, gx, gy, gz);
-    const R rho = mm.rho, ux = mm.ux, uy = mm.uy, uz = mm.uz;
-    const R om1 = R(1) - omega;
-    R s12 = 0, s34 = 0, s56 = 0, q4 = 0, q5 = 0, q6 = 0;
-    R mk[23];                 // MODEL_RATES: moments 4..26 of n
-#pragma unroll
-    for (int k = 0; k < 23; ++k) mk[k] = 0;
-    if constexpr (!bgk && !rates) {
-        const R m4 = ms.m4, m5 = ms.m5, m6 = ms.m6, m7 = ms.m7, m8 = ms.m8;
-        // (1 - omega)(m_k - m_k^eq + R_k / 2), k = 4..8, with the printed m^eq and R
-        const R s4 = m4 - rho * ux * uy + R(0.5) * rho * (gy * ux + gx * uy);
-        const R s5 = m5 - rho * ux * uz + R(0.5) * rho * (gz * ux + gx * uz);
-        const R s6 = m6 - rho * uy * uz + R(0.5) * rho * (gz * uy + gy * uz);
-        const R s7 = m7 - rho * (ux * ux - uy * uy) + rho * (gx * ux - gy * uy);
-        const R s8 = m8 - rho * (ux * ux - uz * uz) + rho * (gx * ux - gz * uz);
-        if (s_out) {
-            s_out[0] = s4; s_out[1] = s5; s_out[2] = s6; s_out[3] = s7; s_out[4] = s8;
-        }
-        const R om1s = SCALED ? om1 * sc : om1;
-        const R a4 = om1s * s4, a5 = om1s * s5, a6 = om1s * s6, a7 = om1s * s7, a8 = om1s * s8;
-        s12 = (a7 + a8) * R(1.0 / 6.0);
-        s34 = a8 * R(1.0 / 6.0) - a7 * R(1.0 / 3.0);
-        s56 = a7 * R(1.0 / 6.0) - a8 * R(1.0 / 3.0);
-        q4 = R(0.25) * a4;
-        q5 = R(0.25) * a5;
-        q6 = R(0.25) * a6;
-    }
-    const R drho = mm.drho;
-    // post-collision value of population i from the equilibrium part pm1 = f^eq / (w rho) - 1
-    // and frc = (1/2) g . grad_u (f^eq / (w rho))
-    auto emit = [&](auto ic, R pm1, R frc) {
-        constexpr int i = decltype(ic)::value;
-        if constexpr (rates) {
-            const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
-            const R ni = v[i] - eq + fh;
-            sfor<4, Q>([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                constexpr int cik = mt_coef(k, i);
-                if constexpr (cik != 0) mk[k - 4] += R(cik) * ni;
-            });
-            v[i] = eq + fh;
-        } else if constexpr (bgk) {
-            const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
-            v[i] = eq + fh + om1 * (v[i] - eq + fh);
-        } else {
-            R f = R(w_of(i)) * (drho + rho * (pm1 + frc));
-            if constexpr (i == 1 || i == 2) f += s12;
-            if constexpr (i == 3 || i == 4) f += s34;
-            if constexpr (i == 5 || i == 6) f += s56;
-            if constexpr (i == 7 || i == 10) f += q4;
-            if constexpr (i == 8 || i == 9) f -= q4;
-            if constexpr (i == 11 || i == 14) f += q5;
-            if constexpr (i == 12 || i == 13) f -= q5;
-            if constexpr (i == 15 || i == 18) f += q6;
-            if constexpr (i == 16 || i == 17) f -= q6;
-            v[i] = f;
-        }
-    };
-    if constexpr (!o2 && !bgk && !rates) {
-        // the default model: f*_i - w_i = w_i drho + w_i rho (pm1 + frc) + shear term, with
-        // pm1 + frc = Dxy + dz axy + Fxy (1 + dz) + hz axy = G + hz axy + dz H per (cx, cy)
-        // column (G = Dxy + Fxy, H = axy + Fxy): three multiply-adds per population
-        R dx[3], hx[3], dy[3], hy[3], dz[3], hz[3];
-        axis_factors<R>(ux, gx, dx, hx);
-        axis_factors<R>(uy, gy, dy, hy);
-        axis_factors<R>(uz, gz, dz, hz);
-        R G[3][3], H[3][3], A[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                const R dxy = dx[a] + dy[b] + dx[a] * dy[b];
-                const R axy = R(1) + dxy;
-                const R fxy = hx[a] * (R(1) + dy[b]) + hy[b] * (R(1) + dx[a]);
-                G[a][b] = dxy + fxy;
-                H[a][b] = axy + fxy;
-                A[a][b] = axy;
-            }
-        // w rho and w drho (plus the shear term of the population) per weight shell
-        R w0 = R(w_of(0)), w1 = R(w_of(1)), w2 = R(w_of(7)), w3 = R(w_of(19));
-        if constexpr (SCALED) {
-            w0 *= sc; w1 *= sc; w2 *= sc; w3 *= sc;
-        }
-        const R wr0 = w0 * rho, wr1 = w1 * rho, wr2 = w2 * rho, wr3 = w3 * rho;
-        const R wd0 = w0 * drho, wd1 = w1 * drho, wd2 = w2 * drho, wd3 = w3 * drho;
-        const R c12 = wd1 + s12, c34 = wd1 + s34, c56 = wd1 + s56;
-        const R c4p = wd2 + q4, c4m = wd2 - q4, c5p = wd2 + q5, c5m = wd2 - q5, c6p = wd2 + q6, c6m = wd2 - q6;
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int a = cx_of(i) + 1, b = cy_of(i) + 1, c = cz_of(i) + 1;
-            const R X = G[a][b] + hz[c] * A[a][b] + dz[c] * H[a][b];
-            R wr, wd;
-            if constexpr (i == 0) { wr = wr0; wd = wd0; }
-            else if constexpr (i <= 6) {
-                wr = wr1;
-                wd = (i <= 2) ? c12 : ((i <= 4) ? c34 : c56);
-            } else if constexpr (i <= 18) {
-                wr = wr2;
-                if constexpr (i == 7 || i == 10) wd = c4p;
-                else if constexpr (i == 8 || i == 9) wd = c4m;
-                else if constexpr (i == 11 || i == 14) wd = c5p;
-                else if constexpr (i == 12 || i == 13) wd = c5m;
-                else if constexpr (i == 15 || i == 18) wd = c6p;
-                else wd = c6m;
-            } else { wr = wr3; wd = wd3; }
-            v[i] = wr * X + wd;
-        });
-    } else if constexpr (!o2) {
-        R dx[3], hx[3], dy[3], hy[3], dz[3], hz[3];
-        axis_factors<R>(ux, gx, dx, hx);
-        axis_factors<R>(uy, gy, dy, hy);
-        axis_factors<R>(uz, gz, dz, hz);
-        // per (cx, cy) pair: Dxy = psi_x psi_y - 1 and the x/y force part
-        R Dxy[3][3], Fxy[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                Dxy[a][b] = dx[a] + dy[b] + dx[a] * dy[b];
-                Fxy[a][b] = hx[a] * (R(1) + dy[b]) + hy[b] * (R(1) + dx[a]);
-            }
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int a = cx_of(i) + 1, b = cy_of(i) + 1, c = cz_of(i) + 1;
-            const R dxy = Dxy[a][b];
-            const R axy = R(1) + dxy;
-            const R pm1 = dxy + dz[c] * axy;                       // psi_x psi_y psi_z - 1
-            const R frc = Fxy[a][b] * (R(1) + dz[c]) + hz[c] * axy; // (1/2) g . grad psi
-            emit(ic, pm1, frc);
-        });
+    const MomentSums<R> ms = moment_sums<R>(v);
+    if constexpr (MODEL == MODEL_MRT_H6) {
+        return collide_mrt<R, SCALED, false, LEAN>(ms, gx, gy, gz, omega, inv, sc, s_out,
+                                      [&](auto ic, R f) { v[decltype(ic)::value] = f; });
     } else {
-        // second-order equilibrium: f^eq / (w rho) - 1 = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u and
-        // (1/2) g . grad_u of it = 3/2 (c.g - u.g) + 9/2 (c.u)(c.g)
-        const R uu = ux * ux + uy * uy + uz * uz, ug = ux * gx + uy * gy + uz * gz;
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int ex = cx_of(i), ey = cy_of(i), ez = cz_of(i);
-            const R cu = cterm<ez>(cterm<ey>(cterm<ex>(R(-0.0), ux), uy), uz);
-            const R cg = cterm<ez>(cterm<ey>(cterm<ex>(R(-0.0), gx), gy), gz);
-            const R pm1 = R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu;
-            const R frc = R(1.5) * (cg - ug) + R(4.5) * cu * cg;
-            emit(ic, pm1, frc);
-        });
-    }
-    if constexpr (rates) {
+        constexpr bool rates = (MODEL & MODEL_RATES) != 0;
+        constexpr bool bgk = !rates && (MODEL & MODEL_BGK) != 0, o2 = (MODEL & MODEL_O2) != 0;
+        const Macro<R> mm = macro_from_sums<R>(ms, R(0.5) * gx, R(0.5) * gy, R(0.5) * gz);
+        const R rho = mm.rho, ux = mm.ux, uy = mm.uy, uz = mm.uz, drho = ms.drho;
+        const R om1 = R(1) - omega;
+        R s12 = 0, s34 = 0, s56 = 0, q4 = 0, q5 = 0, q6 = 0;
+        R mk[23];                 // MODEL_RATES: moments 4..26 of n
 #pragma unroll
-        for (int k = 0; k < 23; ++k) mk[k] *= lam1[k];
-        sfor<0, Q>([&](auto ic) {
+        for (int k = 0; k < 23; ++k) mk[k] = 0;
+        if constexpr (!bgk && !rates) {
+            // (1 - omega)(m_k - m_k^eq + R_k / 2), k = 4..8, with the printed m^eq and R
+            const R a4 = om1 * (ms.m4 - rho * ux * uy + R(0.5) * rho * (gy * ux + gx * uy));
+            const R a5 = om1 * (ms.m5 - rho * ux * uz + R(0.5) * rho * (gz * ux + gx * uz));
+            const R a6 = om1 * (ms.m6 - rho * uy * uz + R(0.5) * rho * (gz * uy + gy * uz));
+            const R a7 = om1 * (ms.m7 - rho * (ux * ux - uy * uy) + rho * (gx * ux - gy * uy));
+            const R a8 = om1 * (ms.m8 - rho * (ux * ux - uz * uz) + rho * (gx * ux - gz * uz));
+            s12 = (a7 + a8) * R(1.0 / 6.0);
+            s34 = a8 * R(1.0 / 6.0) - a7 * R(1.0 / 3.0);
+            s56 = a7 * R(1.0 / 6.0) - a8 * R(1.0 / 3.0);
+            q4 = R(0.25) * a4;
+            q5 = R(0.25) * a5;
+            q6 = R(0.25) * a6;
+        }
+        // post-collision value of population i from the equilibrium part pm1 = f^eq / (w rho) - 1
+        // and frc = (1/2) g . grad_u (f^eq / (w rho))
+        auto emit = [&](auto ic, R pm1, R frc) {
             constexpr int i = decltype(ic)::value;
-            R acc = v[i];
-            sfor<4, Q>([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                constexpr double aik = kMtInv.a[i][k];
-                if constexpr (aik != 0.0) acc += R(aik) * mk[k - 4];
+            if constexpr (rates) {
+                const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
+                const R ni = v[i] - eq + fh;
+                sfor<4, Q>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    constexpr int cik = mt_coef(k, i);
+                    if constexpr (cik != 0) mk[k - 4] += R(cik) * ni;
+                });
+                v[i] = eq + fh;
+            } else if constexpr (bgk) {
+                const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
+                v[i] = eq + fh + om1 * (v[i] - eq + fh);
+            } else {
+                R f = R(w_of(i)) * (drho + rho * (pm1 + frc));
+                if constexpr (i == 1 || i == 2) f += s12;
+                if constexpr (i == 3 || i == 4) f += s34;
+                if constexpr (i == 5 || i == 6) f += s56;
+                if constexpr (i == 7 || i == 10) f += q4;
+                if constexpr (i == 8 || i == 9) f -= q4;
+                if constexpr (i == 11 || i == 14) f += q5;
+                if constexpr (i == 12 || i == 13) f -= q5;
+                if constexpr (i == 15 || i == 18) f += q6;
+                if constexpr (i == 16 || i == 17) f -= q6;
+                v[i] = f;
+            }
+        };
+        if constexpr (!o2) {
+            R dx[3], hx[3], dy[3], hy[3], dz[3], hz[3];
+            axis_factors<R>(ux, gx, dx, hx);
+            axis_factors<R>(uy, gy, dy, hy);
+            axis_factors<R>(uz, gz, dz, hz);
+            // per (cx, cy) pair: Dxy = psi_x psi_y - 1 and the x/y force part
+            R Dxy[3][3], Fxy[3][3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    Dxy[a][b] = dx[a] + dy[b] + dx[a] * dy[b];
+                    Fxy[a][b] = hx[a] * (R(1) + dy[b]) + hy[b] * (R(1) + dx[a]);
+                }
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                constexpr int a = cx_of(i) + 1, b = cy_of(i) + 1, c = cz_of(i) + 1;
+                const R dxy = Dxy[a][b];
+                const R axy = R(1) + dxy;
+                const R pm1 = dxy + dz[c] * axy;                       // psi_x psi_y psi_z - 1
+                const R frc = Fxy[a][b] * (R(1) + dz[c]) + hz[c] * axy; // (1/2) g . grad psi
+                emit(ic, pm1, frc);
             });
-            v[i] = acc;
-        });
+        } else {
+            // second-order equilibrium: f^eq / (w rho) - 1 = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u and
+            // (1/2) g . grad_u of it = 3/2 (c.g - u.g) + 9/2 (c.u)(c.g)
+            const R uu = ux * ux + uy * uy + uz * uz, ug = ux * gx + uy * gy + uz * gz;
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                constexpr int ex = cx_of(i), ey = cy_of(i), ez = cz_of(i);
+                const R cu = cterm<ez>(cterm<ey>(cterm<ex>(R(-0.0), ux), uy), uz);
+                const R cg = cterm<ez>(cterm<ey>(cterm<ex>(R(-0.0), gx), gy), gz);
+                const R pm1 = R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu;
+                const R frc = R(1.5) * (cg - ug) + R(4.5) * cu * cg;
+                emit(ic, pm1, frc);
+            });
+        }
+        if constexpr (rates) {
+#pragma unroll
+            for (int k = 0; k < 23; ++k) mk[k] *= lam1[k];
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                R acc = v[i];
+                sfor<4, Q>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    constexpr double aik = kMtInv.a[i][k];
+                    if constexpr (aik != 0.0) acc += R(aik) * mk[k - 4];
+                });
+                v[i] = acc;
+            });
+        }
+        return mm;
     }
-    return mm;
 }
 
 }  // namespace lbm

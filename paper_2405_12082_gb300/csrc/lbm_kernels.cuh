@@ -49,7 +49,7 @@ __device__ __forceinline__ void finish_cell(const StepArgs &a, const Member &d, 
         for (int k = 0; k < 5; ++k) mo[(4 + k) * n] = sk[k];
     } else {
         constexpr bool SC = Storage<P>::kScaled && MODEL == MODEL_MRT_H6;
-        const Macro<R> mm = collide<R, MODEL, SC>(v, gx, gy, gz, omega_of<R>(d), nullptr, lam1_of<R>(d),
+        const Macro<R> mm = collide<R, MODEL, SC, P != LBM_F32>(v, gx, gy, gz, omega_of<R>(d), nullptr, lam1_of<R>(d),
                                                   (R)a.f16_inv, (R)a.f16_scale);
         if constexpr (EXTRA == EX_STATS) {
             const double uz = (double)mm.uz;
