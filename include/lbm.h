@@ -258,12 +258,14 @@ int lbm_set_graph(lbm_ctx *ctx, int32_t chunk);
  * blocks per SM; 1 = 256 x 3; 2 = 128 x 8; 3 = 512 x 2; for LBM_F32 also the
  * software-pipelined persistent kernel, 4 = 256 x 3 and 5 = 128 x 6 (each thread
  * copies its next cell's 27 populations into shared memory with cp.async while it
- * computes the current one); 6 = 128 x 8 with each thread taking 2 consecutive planes
- * of one in-plane position (the default for F32 storage), 7 = the same with 4 planes
- * (the default for the 16-bit formats and for LBM_BOUZIDI walls), 8 = 256 x 4, 9 = 128 x 7 and 10 = 128 x 6 with 2
- * planes; 11 and 12 = the staged persistent kernel (512 threads with 3 tiles in flight,
- * one CTA per SM; 256 threads, 3 tiles, two CTAs per SM): a tile is a group of whole
- * fluid rows of one plane, whose populations the kernel copies into shared memory with
+ * computes the current one); 6-10 = several planes per thread: 128 x 8 with 2
+ * and with 4 planes, 256 x 4, 128 x 7 and 128 x 6 with 2 (full-way walls, periodic box); on
+ * pipes with half-way or Bouzidi walls in LBM_F32 and the 16-bit formats these run on pairs
+ * of cells with the paired FP32 instructions, even steps 128 x 5 on neighbours in x, odd
+ * steps on neighbours in z: 6 = 256 x 2 and 9 = 128 x 4 with 2 planes per thread, 7 = 128 x 4
+ * and 8 = 64 x 8 with 4, 10 = 128 x 4 with 8; 11 and 12 = the staged persistent kernel (512
+ * threads with 3 tiles in flight, one CTA per SM; 256 threads, 3 tiles, two CTAs per SM): a
+ * tile is a group of whole fluid rows of one plane, whose populations the kernel copies with
  * bulk copies (cp.async.bulk, completing on an mbarrier) several tiles ahead, so loads
  * are in flight without holding registers; available in every storage for pipes with
  * half-way or Bouzidi walls whose rows fit its shared-memory segments.  LBM_F64 has shape
@@ -276,8 +278,9 @@ int lbm_set_variant(lbm_ctx *ctx, int32_t variant);
 
 /* Launch shapes per parity of the AA pattern: `even` for the steps with even t (own
  * slots), `odd` for the others (neighbour slots); lbm_set_variant sets both.  The defaults
- * are the fastest pair measured on GB300 (F32: 6 even, 9 odd; 16-bit formats: 7 and 9;
- * Bouzidi walls: 7 and 7; F64: 0 and 0).  Same errors as lbm_set_variant. */
+ * are the fastest pair measured on GB300 (F32: 6 even, 9 odd; 16-bit formats and Bouzidi
+ * walls: 7 even and, from about 10 M stored cells on, 7 odd, else 9; F64: 0 and 0).  Same
+ * errors as lbm_set_variant. */
 int lbm_set_variants(lbm_ctx *ctx, int32_t even, int32_t odd);
 
 /* Failure-detection tests of the staged shapes (11, 12): the next step launched directly

@@ -193,6 +193,7 @@ std::vector<int4> row_groups(const Member &d, const std::vector<int32_t> &rows, 
 int build_tables(lbm_ctx *c) {
     const size_t es = c->precision == LBM_F64 ? 8 : 4;
     std::vector<size_t> at(c->hm.size() * 3), at_rows(c->hm.size()), at_delta(c->hm.size());
+    std::vector<size_t> at_pair(c->hm.size());
     std::vector<size_t> at_sg(c->hm.size() * 2);
     std::vector<std::vector<int4>> sg(c->hm.size() * 2);
     size_t total = 0;
@@ -205,6 +206,8 @@ int build_tables(lbm_ctx *c) {
                      align256(c->rowof[m].size() * sizeof(int4));
         at[3 * m] = total; total += align256(ncol * 2);
         at[3 * m + 1] = total; total += align256(3 * ncol * es);
+        at_pair[m] = total;
+        if (d.compact) total += align256((size_t)d.Ps / 2 * 4) + align256(3 * (size_t)d.Ps * es);
         at[3 * m + 2] = total; total += align256(2 * (size_t)d.nz * es);
         at_delta[m] = total;
         if (c->wall == LBM_BOUZIDI) total += align256(27 * ncol * es);
@@ -259,6 +262,19 @@ int build_tables(lbm_ctx *c) {
             char *gi = g + at_rows[m] + align256(rb) + align256(ro.size() * 2);
             LBM_CUDA(c, cudaMemcpy(gi, info.data(), info.size() * sizeof(int4), cudaMemcpyHostToDevice));
             d.cellinfo = (const int4 *)gi;
+            std::vector<uint32_t> pi(ro.size() / 2, 0);
+            for (size_t k = 0; k < pi.size(); ++k) {
+                const int4 A = info[2 * k], B = info[2 * k + 1];
+                if (A.x == -1) continue;                    // a row's cells come before its padding
+                const uint32_t x = (uint32_t)A.x >> 16, y = (uint32_t)A.x & 0xFFFF;
+                pi[k] = ((y * (uint32_t)d.nx + x) << lbm::PAIR_SHIFT) | lbm::PAIR_A;
+                if (B.x != -1) pi[k] |= lbm::PAIR_B;
+                if (A.y != 0x1FF || (B.x != -1 && B.y != 0x1FF)) pi[k] |= lbm::PAIR_WALL;
+            }
+            LBM_CUDA(c, cudaMemcpy(g + at_pair[m], pi.data(), pi.size() * 4, cudaMemcpyHostToDevice));
+            d.pairinfo = (const uint32_t *)(g + at_pair[m]);
+            d.ftabc = g + at_pair[m] + align256(pi.size() * 4);
+            LBM_CUDA(c, cudaMemset(const_cast<void *>(d.ftabc), 0, 3 * (size_t)d.Ps * es));
         }
         for (int k = 0; k < 2; ++k) {
             const std::vector<int4> &grp = sg[2 * m + k];
@@ -403,7 +419,7 @@ int update_collision(lbm_ctx *c) {
     if (code != c->collision) {
         c->collision = code;
         c->variant = code != 0 ? model_variant(c->precision) : default_variant(c->precision, c->wall);
-        c->variant_odd = code != 0 ? model_variant(c->precision) : default_variant_odd(c->precision, c->wall);
+        c->variant_odd = code != 0 ? model_variant(c->precision) : default_variant_odd(c->precision, c->wall, c->stride);
         drop_graph(c);
     }
     return LBM_OK;
@@ -482,6 +498,16 @@ int build_member(lbm_ctx *c, const lbm_grid *g, const lbm_relax *r, const lbm_fo
 // Launch shape of the step with index t.
 int variant_at(const lbm_ctx *c, int64_t t) { return (t & 1) ? c->variant_odd : c->variant; }
 
+// Whether the even steps of the shapes of several planes per thread run on pairs of cells
+// (lbm_pair.cuh): F32 or 16-bit storage, the default model, every member compact and its
+// columns within the pair table's index range.
+bool pairs_of(const lbm_ctx *c) {
+    if (c->precision == LBM_F64 || c->collision != 0) return false;
+    for (const Member &d : c->hm)
+        if (!d.compact || (int64_t)d.nx * d.ny >= (1ll << (32 - lbm::PAIR_SHIFT))) return false;
+    return true;
+}
+
 StepArgs make_args(const lbm_ctx *c, int64_t t) {
     StepArgs a;
     std::memset(&a, 0, sizeof a);
@@ -496,8 +522,7 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
     a.dstride = c->dense_total;
     a.collision = c->collision;
     const int v = variant_at(c, t);
-    const int bs = lbm::step_threads(c->precision, v);
-    const int zc = lbm::step_zc(c->precision, v);
+    int bs = lbm::step_threads(c->precision, v), zc = lbm::step_zc(c->precision, v);
     const int sk = lbm::staged_of(v);
     a.err = c->flags;
     a.skip_tile = -1;
@@ -506,6 +531,9 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         a.sg_sel = sk;
     }
     int64_t blk = 0;
+    const bool pairs = zc > 1 && pairs_of(c);
+    a.pairs = pairs;
+    if (zc > 1 && !pairs && c->wall == LBM_BOUZIDI) bs = 128, zc = 1;      // see launch_planes
     for (size_t m = 0; m < c->hm.size(); ++m) {
         const Member &d = c->hm[m];
         a.st[m] = (d.trig && t < d.t_end) ? std::sin(2.0 * M_PI * (double)t / d.period) : 0.0;
@@ -513,6 +541,11 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         a.block0[m] = (int32_t)blk;
         if (sk >= 0) {
             blk += (int64_t)d.nsg[sk] * d.nz;        // staged: one tile per (plane, row group)
+        } else if (pairs && (t & 1) == 0) {
+            blk += ceil_div(d.scells / 2, 128);      // pairs of stored positions
+        } else if (pairs) {
+            blk += ceil_div(d.Ps, lbm::STEP_SHAPES[v].pt) *
+                   (lbm::odd_single_planes(d.nz) + lbm::odd_pair_groups(d.nz, lbm::STEP_SHAPES[v].pz));
         } else {
             // threads over (plane group, in-plane position); zc = 1 is every stored cell
             const int64_t work = (int64_t)d.Ps * ((d.nz + zc - 1) / zc);
@@ -586,7 +619,6 @@ int create_common(lbm_ctx **out, int32_t n, const lbm_grid *grids, const lbm_rel
     c->precision = prec;
     c->wall = wall;
     c->variant = default_variant(prec, wall);
-    c->variant_odd = lbm::default_variant_odd(prec, wall);
     c->stream = (cudaStream_t)stream;
     c->f16_scale = std::ldexp(1.0f, s16);
     c->f16_inv = std::ldexp(1.0f, -s16);
@@ -622,6 +654,7 @@ int create_common(lbm_ctx **out, int32_t n, const lbm_grid *grids, const lbm_rel
                        "27 x %lld cells exceed the 32-bit population index of the step kernels", (long long)off);
     }
     c->stride = off;
+    c->variant_odd = default_variant_odd(prec, wall, off);
     c->dense_total = doff;
     c->esize = esize_of(prec);
     c->mass0.assign(n, 0.0);
@@ -987,8 +1020,8 @@ int step_direct(lbm_ctx *c) {
         LBM_CUDA(c, cudaEventRecord(e0, c->stream));
     }
     int rc = dispatch(c, [&](auto P) {
-        return lbm::launch_step<decltype(P)::value>(c->wall, (int)(c->t & 1), stats, a, variant_at(c, c->t),
-                                                    c->stream);
+        return lbm::launch_step<decltype(P)::value>(c->wall, (int)(c->t & 1), stats, a, c->hm.data(),
+                                                    variant_at(c, c->t), c->stream);
     });
     if (rc) return rc;
     if (c->prof) {
@@ -1033,10 +1066,10 @@ int build_graph(lbm_ctx *c) {
         const bool stats = every > 0 && (k % every == 0);
         const int v = variant_at(c, k);
         switch (c->precision) {
-            case LBM_F64: le = lbm::launch_step<LBM_F64>(c->wall, k & 1, stats, a, v, cs); break;
-            case LBM_F32: le = lbm::launch_step<LBM_F32>(c->wall, k & 1, stats, a, v, cs); break;
-            case LBM_F16S: le = lbm::launch_step<LBM_F16S>(c->wall, k & 1, stats, a, v, cs); break;
-            default: le = lbm::launch_step<LBM_BF16>(c->wall, k & 1, stats, a, v, cs); break;
+            case LBM_F64: le = lbm::launch_step<LBM_F64>(c->wall, k & 1, stats, a, c->hm.data(), v, cs); break;
+            case LBM_F32: le = lbm::launch_step<LBM_F32>(c->wall, k & 1, stats, a, c->hm.data(), v, cs); break;
+            case LBM_F16S: le = lbm::launch_step<LBM_F16S>(c->wall, k & 1, stats, a, c->hm.data(), v, cs); break;
+            default: le = lbm::launch_step<LBM_BF16>(c->wall, k & 1, stats, a, c->hm.data(), v, cs); break;
         }
     }
     cudaGraph_t g = nullptr;

@@ -9,6 +9,76 @@
 
 namespace lbm {
 
+// What else a step does: EX_STATS adds u_z^k of the pre-collision state to the FP64 sums,
+// EX_MOMENTS stores the adjoint's moments.
+enum { EX_NONE = 0, EX_STATS = 1, EX_MOMENTS = 2 };
+
+// FP64 sums of u_z^k, k = 1..4, of one cell (stride between the four sums); single roundings,
+// so every kernel adds the same bits.
+__device__ __forceinline__ void add_stats(double *s, int64_t stride, double uz) {
+    const double uz2 = __dmul_rn(uz, uz);
+    s[0] = __dadd_rn(s[0], uz);
+    s[stride] = __dadd_rn(s[stride], uz2);
+    s[2 * stride] = __fma_rn(uz2, uz, s[2 * stride]);
+    s[3 * stride] = __fma_rn(uz2, uz2, s[3 * stride]);
+}
+
+// Kernel parameters of the pair kernels (lbm_pair.cuh): a single pipe carries its member in
+// the parameters, an ensemble its block table.
+struct PairMember {
+    const uint32_t *pairinfo;
+    const int4 *cellinfo;
+    const void *ftabc, *ztab, *dtab, *gz_field;
+    int64_t off, doff, scells, t_end;
+    int32_t nx, ny, nz, Ps, trig;
+    uint32_t ps_mul, ps_shr;
+    float gf[3], omegaf;
+};
+struct PairArgsBase {
+    void *pops;
+    int64_t stride;
+    const StepTime *times;
+    int64_t t;
+    double *stats;
+    int64_t dstride;
+    int32_t tidx;
+    float f16_scale, f16_inv;
+    uint32_t zero;           // 0 (see k_odd2)
+};
+struct PairArgsOne : PairArgsBase {
+    static constexpr bool kOne = true;
+    float stf[1];
+    uint32_t nb_plane, nb_mul, nb_shr;
+    uint32_t own[27], pull[27];
+    PairMember one;
+};
+struct PairArgsMany : PairArgsBase {
+    static constexpr bool kOne = false;
+    const Member *members;
+    int32_t n_members;
+    float stf[LBM_MAX_MEMBERS];
+    int32_t block0[LBM_MAX_MEMBERS + 1];
+};
+// Resident blocks of 128 threads the even pair kernel's registers are cut for (5: 96 registers).
+// R = 96 / R = 48 pipe, fraction of the copy bandwidth: F32 5 blocks 0.992 / 0.907 (4: 0.987 /
+// 0.897, 6: 0.963 / 0.876), F16S 0.773 / 0.659 (4: 0.70 / 0.61), BF16 0.715 / 0.607.
+constexpr int EVEN2_BLOCKS = 5;
+// Planes the odd pair kernel takes singly (0, nz - 1 and, for odd nz > 2, nz - 2), and its plane
+// groups of zc planes (the pairs 1 .. nz - 2) after them.
+__host__ __device__ inline int odd_single_planes(int nz) { return nz < 3 ? nz : 2 + (nz & 1); }
+__host__ __device__ inline int odd_pair_groups(int nz, int zc) { return nz < 3 ? 0 : ((nz - 2) / 2 * 2 + zc - 1) / zc; }
+inline void fill_pair_args(PairArgsBase &o, const StepArgs &a) {
+    o.pops = a.pops; o.stride = a.stride; o.times = a.times; o.t = a.t; o.stats = a.stats; o.dstride = a.dstride;
+    o.tidx = a.tidx; o.zero = 0; o.f16_scale = a.f16_scale; o.f16_inv = a.f16_inv;
+}
+inline void fill_pair_member(PairMember &o, const Member &d) {
+    o.pairinfo = d.pairinfo; o.cellinfo = d.cellinfo; o.ftabc = d.ftabc; o.ztab = d.ztab; o.dtab = d.dtab;
+    o.gz_field = d.gz_field; o.off = d.off; o.doff = d.doff; o.scells = d.scells; o.t_end = d.t_end;
+    o.nx = d.nx; o.ny = d.ny; o.nz = d.nz; o.Ps = d.Ps; o.trig = d.trig; o.ps_mul = d.ps_mul; o.ps_shr = d.ps_shr;
+    for (int k = 0; k < 3; ++k) o.gf[k] = d.gf[k];
+    o.omegaf = d.omegaf;
+}
+
 struct ModesArgs {
     int32_t n_sections, n_rings, n_theta, n_modes;
     double r_over_R[16];
@@ -20,11 +90,20 @@ struct ModesArgs {
 // storage only) and whether it is the persistent kernel whose loads are staged in shared
 // memory by bulk copies (shapes 11 and 12, compact pipe layouts, every storage; staged =
 // index into STAGED_SHAPES + 1).  FP64 storage has shape 0 (256 x 2) and the staged ones.
-struct StepShape { int threads, min_blocks, zc, pipelined, staged; };
-constexpr StepShape STEP_SHAPES[13] = {{256, 4, 1, 0, 0}, {256, 3, 1, 0, 0}, {128, 8, 1, 0, 0}, {512, 2, 1, 0, 0},
-                                       {256, 3, 1, 1, 0}, {128, 6, 1, 1, 0}, {128, 8, 2, 0, 0}, {128, 8, 4, 0, 0},
-                                       {256, 4, 2, 0, 0}, {128, 7, 2, 0, 0}, {128, 6, 2, 0, 0}, {992, 1, 1, 0, 1},
-                                       {512, 1, 1, 0, 2}};
+// Shapes 6-10 (several planes per thread) run on pairs of cells in the compact pipe layouts
+// (lbm_pair.cuh): pt, pb, pz are the threads, resident blocks and planes per thread of their
+// odd steps there; zc, threads and min_blocks hold for the dense layouts.
+// Odd steps, measured on the R = 96 / R = 48 pipes: 128 threads x 4 blocks (128 registers, no
+// spills) 1176 / 131 us in F32 with 2 planes per thread, 1187 / 138 us with 4 (the last wave of
+// blocks is longer); 128 x 5 spills and takes 1305 / 150 us, 256 x 2 takes 1211 / 138.  F16S:
+// 894 / 101 us with 2 planes, 866 / 104 with 4; BF16 891 / 101 and 866 / 105.  Bouzidi walls in
+// F32: 1364 / 151 us with 2 planes, 1293 / 151 with 4 (fewer loads of the link coefficients).
+struct StepShape { int threads, min_blocks, zc, pipelined, staged, pt, pb, pz; };
+constexpr StepShape STEP_SHAPES[13] = {{256, 4, 1, 0, 0, 0, 0, 0},    {256, 3, 1, 0, 0, 0, 0, 0},   {128, 8, 1, 0, 0, 0, 0, 0},
+                                       {512, 2, 1, 0, 0, 0, 0, 0},    {256, 3, 1, 1, 0, 0, 0, 0},   {128, 6, 1, 1, 0, 0, 0, 0},
+                                       {128, 8, 2, 0, 0, 256, 2, 2},  {128, 8, 4, 0, 0, 128, 4, 4}, {256, 4, 2, 0, 0, 64, 8, 4},
+                                       {128, 7, 2, 0, 0, 128, 4, 2},  {128, 6, 2, 0, 0, 128, 4, 8}, {992, 1, 1, 0, 1, 0, 0, 0},
+                                       {512, 1, 1, 0, 2, 0, 0, 0}};
 constexpr StepShape STEP_SHAPE_F64 = {256, 2, 1, 0, 0};
 constexpr int N_STEP_SHAPES = 13;
 // Staged shapes: threads per CTA (one producer warp, the rest consume), pipeline stages
@@ -48,21 +127,18 @@ inline int staged_cap(int precision, int k) {
     return budget / per / 64 * 64;
 }
 inline int step_variants(int) { return N_STEP_SHAPES; }
-// the fastest shapes in sweeps on GB300: 128 x 8 threads with 2 planes per thread for
-// F32 storage, with 4 planes for the 16-bit formats and for Bouzidi walls (with the link
-// coefficients tabulated per wall link, 4 planes per thread beat one by 4 %)
+// the fastest shapes in sweeps on GB300 (see STEP_SHAPES; even steps run the same pair kernel
+// in shapes 6-10).  Odd steps of the 16-bit formats and of Bouzidi walls: 4 planes per thread
+// on large contexts, 2 below about 10 M stored cells, where 4 leave too few waves of blocks
+// (F16S: R = 96 pipe, 36 M cells, 866 against 894 us; R = 48 pipe, 3.9 M, 104 against 101 us).
 inline int default_variant(int precision, int wall) {
     if (precision == LBM_F64) return 0;
     if (wall == LBM_BOUZIDI) return 7;
     return precision == LBM_F32 ? 6 : 7;
 }
-// the fastest shape of the odd (neighbour-slot) steps: 128 x 7 with 2 planes per thread
-// (more registers for the 27 neighbour addresses and wall-link selects; R = 96 pipe: odd
-// step 0.855 of measured HBM against 0.824 with the even steps' shape)
-inline int default_variant_odd(int precision, int wall) {
+inline int default_variant_odd(int precision, int wall, int64_t stored_cells) {
     if (precision == LBM_F64) return 0;
-    if (wall == LBM_BOUZIDI) return 7;
-    return 9;
+    return (wall == LBM_BOUZIDI || precision != LBM_F32) && stored_cells >= 10000000 ? 7 : 9;
 }
 // the shape the ablation collision models are compiled for (one plane per thread)
 inline int model_variant(int precision) { return precision == LBM_F64 ? 0 : 2; }
@@ -97,7 +173,8 @@ cudaError_t launch_step_staged(int wall, int parity, bool stats, const StepArgs 
 // Step kernel over all members: a flat grid of a.nblocks_total blocks of
 // step_threads(P, variant) threads.
 template <int P>
-cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, int variant, cudaStream_t s);
+cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, int variant,
+                        cudaStream_t s);
 
 // Forward step that also stores rho, u, s4..s8 into a.moments (adjoint recompute;
 // single half-way pipe, F32 or F64 storage, in the shape moments_variant).

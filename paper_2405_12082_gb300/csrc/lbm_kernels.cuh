@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "lbm_internal.h"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 
@@ -16,7 +17,6 @@ namespace lbm {
 // the FP64 sums (sample steps); EX_MOMENTS stores rho, u and s4..s8 of the
 // pre-collision state for the adjoint sweep.  BS threads per block, register budget
 // for MINB resident blocks per SM.
-enum { EX_NONE = 0, EX_STATS = 1, EX_MOMENTS = 2 };
 #ifndef LBM_ADJ_MIN_BLOCKS
 #define LBM_ADJ_MIN_BLOCKS 3
 #endif
@@ -53,12 +53,7 @@ __device__ __forceinline__ void finish_cell(const StepArgs &a, const Member &d, 
                                                   (R)a.f16_inv, (R)a.f16_scale);
         if constexpr (EXTRA == EX_STATS) {
             const double uz = (double)mm.uz;
-            double *s = a.stats + d.doff + p.di;
-            const double uz2 = uz * uz;
-            s[0] += uz;
-            s[a.dstride] += uz2;
-            s[2 * a.dstride] += uz2 * uz;
-            s[3 * a.dstride] += uz2 * uz2;
+            add_stats(a.stats + d.doff + p.di, a.dstride, uz);
         }
     }
     store_pops<P, PAR, WALL, raw_units<P, EXTRA, MODEL>()>(a, d, p, v);
@@ -218,12 +213,7 @@ __global__ void __launch_bounds__(BS, MINB) k_step_pipe(const __grid_constant__ 
             const Macro<R> mm = collide<R>(v, gx, gy, gz, omega_of<R>(d));
             if constexpr (EXTRA == EX_STATS) {
                 const double uz = (double)mm.uz;
-                double *sp = a.stats + d.doff + cur.p.di;
-                const double uz2 = uz * uz;
-                sp[0] += uz;
-                sp[a.dstride] += uz2;
-                sp[2 * a.dstride] += uz2 * uz;
-                sp[3 * a.dstride] += uz2 * uz2;
+                add_stats(a.stats + d.doff + cur.p.di, a.dstride, uz);
             }
             store_pops<P, PAR, WALL>(a, d, cur.p, v);
         }
@@ -568,6 +558,13 @@ __global__ void k_force_tables(const Member *members, int m, R *ftab, R *ztab) {
         ftab[k] = (R)Px;
         ftab[ncol + k] = (R)Py;
         ftab[2 * ncol + k] = (R)Pz;
+        if (d.compact && ((d.colmask[k] >> 4) & 1u)) {       // the same by stored position
+            const int y = k / d.nx, x = k % d.nx;
+            R *fc = static_cast<R *>(const_cast<void *>(d.ftabc)) + (d.rowbase[y] + x - d.rowx0[y]);
+            fc[0] = (R)Px;
+            fc[d.Ps] = (R)Py;
+            fc[2 * (int64_t)d.Ps] = (R)Pz;
+        }
     }
     if (k < d.nz) {
         double sz, cz;
@@ -924,8 +921,71 @@ cudaError_t launch_step_model(int wall, int parity, bool stats, const StepArgs &
     return cudaGetLastError();
 }
 
+// A step of a compact pipe context on pairs of cells, in shape V.
+template <int P, int V, int WALL, class A>
+cudaError_t launch_pair_args(int parity, bool stats, int blocks, const A &a, cudaStream_t s) {
+    constexpr StepShape S = STEP_SHAPES[V];
+    if (parity == 0) {
+        if (stats) k_even2<P, WALL, EX_STATS, 128, EVEN2_BLOCKS, A><<<blocks, 128, 0, s>>>(a);
+        else k_even2<P, WALL, EX_NONE, 128, EVEN2_BLOCKS, A><<<blocks, 128, 0, s>>>(a);
+    } else {
+        if (stats) k_odd2<P, WALL, EX_STATS, S.pt, S.pb, S.pz, A><<<blocks, S.pt, 0, s>>>(a);
+        else k_odd2<P, WALL, EX_NONE, S.pt, S.pb, S.pz, A><<<blocks, S.pt, 0, s>>>(a);
+    }
+    return cudaGetLastError();
+}
+
+template <int P, int V>
+cudaError_t launch_pair(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, cudaStream_t s) {
+    if (a.n_members == 1) {
+        PairArgsOne o;
+        fill_pair_args(o, a);
+        fill_pair_member(o.one, hm[0]);
+        o.stf[0] = a.stf[0];
+        o.nb_plane = (uint32_t)((hm[0].Ps + STEP_SHAPES[V].pt - 1) / STEP_SHAPES[V].pt);
+        fastdiv_setup(o.nb_plane, o.nb_mul, o.nb_shr);
+        for (int i = 0; i < Q; ++i) {
+            o.own[i] = (uint32_t)i * (uint32_t)a.stride;
+            o.pull[i] = (uint32_t)(opp_of(i) - i) * (uint32_t)a.stride - (uint32_t)(cz_of(i) * hm[0].Ps);
+        }
+        return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, o, s)
+                                   : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, o, s);
+    }
+    PairArgsMany o;
+    fill_pair_args(o, a);
+    o.members = a.members;
+    o.n_members = a.n_members;
+    for (int m = 0; m < a.n_members; ++m) o.stf[m] = a.stf[m];
+    for (int m = 0; m <= a.n_members; ++m) o.block0[m] = a.block0[m];
+    return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, o, s)
+                               : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, o, s);
+}
+
+// A shape of several planes per thread: pairs of cells in the compact pipe layouts, else
+// (full-way walls, periodic box) the planes one after the other.
+template <int P, int V>
+cudaError_t launch_planes(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, cudaStream_t s) {
+    if (a.pairs) return launch_pair<P, V>(wall, parity, stats, a, hm, s);
+    constexpr StepShape S = STEP_SHAPES[V];
+    // (a pipe too wide for the pair tables: its Bouzidi walls run one plane per thread)
+    if (wall == LBM_BOUZIDI) return launch_step_shape<P, 128, 8>(wall, parity, stats, a, s);
+    const bool full = wall == LBM_FULLWAY;
+    auto go = [&](auto pa, auto w) {
+        constexpr int PA = decltype(pa)::value, W = decltype(w)::value;
+        if (stats) k_step<P, PA, W, EX_STATS, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc><<<a.nblocks_total, S.threads, 0, s>>>(a);
+        else k_step<P, PA, W, EX_NONE, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc><<<a.nblocks_total, S.threads, 0, s>>>(a);
+    };
+    using std::integral_constant;
+    if (full && parity == 0) go(integral_constant<int, 0>{}, integral_constant<int, LBM_FULLWAY>{});
+    else if (full) go(integral_constant<int, 1>{}, integral_constant<int, LBM_FULLWAY>{});
+    else if (parity == 0) go(integral_constant<int, 0>{}, integral_constant<int, LBM_HALFWAY>{});
+    else go(integral_constant<int, 1>{}, integral_constant<int, LBM_HALFWAY>{});
+    return cudaGetLastError();
+}
+
 template <int P>
-cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, int variant, cudaStream_t s) {
+cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, int variant,
+                        cudaStream_t s) {
     if (a.nblocks_total <= 0) return cudaSuccess;
     if (a.collision == MODEL_MRT_H6 && STEP_SHAPES[variant].staged)
         return launch_step_staged<P>(wall, parity, stats, a, variant, s);
@@ -947,11 +1007,11 @@ cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, int
             case 5:
                 if constexpr (P == LBM_F32) return launch_step_pipe<P, 128, 6>(wall, parity, stats, a, s);
                 else return cudaErrorInvalidValue;
-            case 6: return launch_step_shape<P, STEP_SHAPES[6].threads, STEP_SHAPES[6].min_blocks, STEP_SHAPES[6].zc>(wall, parity, stats, a, s);
-            case 7: return launch_step_shape<P, STEP_SHAPES[7].threads, STEP_SHAPES[7].min_blocks, STEP_SHAPES[7].zc>(wall, parity, stats, a, s);
-            case 8: return launch_step_shape<P, STEP_SHAPES[8].threads, STEP_SHAPES[8].min_blocks, STEP_SHAPES[8].zc>(wall, parity, stats, a, s);
-            case 9: return launch_step_shape<P, STEP_SHAPES[9].threads, STEP_SHAPES[9].min_blocks, STEP_SHAPES[9].zc>(wall, parity, stats, a, s);
-            case 10: return launch_step_shape<P, STEP_SHAPES[10].threads, STEP_SHAPES[10].min_blocks, STEP_SHAPES[10].zc>(wall, parity, stats, a, s);
+            case 6: return launch_planes<P, 6>(wall, parity, stats, a, hm, s);
+            case 7: return launch_planes<P, 7>(wall, parity, stats, a, hm, s);
+            case 8: return launch_planes<P, 8>(wall, parity, stats, a, hm, s);
+            case 9: return launch_planes<P, 9>(wall, parity, stats, a, hm, s);
+            case 10: return launch_planes<P, 10>(wall, parity, stats, a, hm, s);
             default: return launch_step_shape<P, 256, 4>(wall, parity, stats, a, s);
         }
     }
@@ -1087,7 +1147,8 @@ cudaError_t launch_modes(int wall, int parity, const StepArgs &a, const Member &
 // Explicit instantiation of every launcher for one storage precision.
 #define LBM_INSTANTIATE(P)                                                                              \
     namespace lbm {                                                                                     \
-    template cudaError_t launch_step<P>(int, int, bool, const StepArgs &, int, cudaStream_t);           \
+    template cudaError_t launch_step<P>(int, int, bool, const StepArgs &, const Member *, int,            \
+                                         cudaStream_t);                                                  \
     template cudaError_t launch_step_moments<P>(int, const StepArgs &, cudaStream_t);                    \
     template cudaError_t launch_adjoint<P>(const StepArgs &, const AdjArgs &, cudaStream_t);             \
     template cudaError_t launch_flush_segment<P>(const StepArgs &, const Member &, const AdjArgs &,       \
