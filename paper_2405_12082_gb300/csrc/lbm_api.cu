@@ -56,6 +56,7 @@ struct lbm_ctx {
     int64_t launches = 0;
     int variant = 0;                 // launch shape of the step kernel at even t
     int variant_odd = 0;             // ... and at odd t
+    bool shape_set = false;          // the caller or the autotuner chose them
     int collision = 0;               // collision model of the step kernel (lbm::MODEL_* bits)
     int model_bits = 0;              // lbm_set_collision: MODEL_BGK, MODEL_O2
     std::vector<bool> has_rates;     // per member: a general relaxation matrix was given
@@ -207,6 +208,7 @@ int build_tables(lbm_ctx *c) {
         at[3 * m] = total; total += align256(ncol * 2);
         at[3 * m + 1] = total; total += align256(3 * ncol * es);
         at_pair[m] = total;
+        if (d.geometry == LBM_PIPE && !d.compact) total += align256((size_t)std::max(d.Pw, 1) * 4);
         if (d.compact) total += align256((size_t)d.Ps / 2 * 4) + align256(3 * (size_t)d.Ps * es);
         at[3 * m + 2] = total; total += align256(2 * (size_t)d.nz * es);
         at_delta[m] = total;
@@ -275,6 +277,14 @@ int build_tables(lbm_ctx *c) {
             d.pairinfo = (const uint32_t *)(g + at_pair[m]);
             d.ftabc = g + at_pair[m] + align256(pi.size() * 4);
             LBM_CUDA(c, cudaMemset(const_cast<void *>(d.ftabc), 0, 3 * (size_t)d.Ps * es));
+        }
+        d.fluidcol = nullptr;
+        if (d.geometry == LBM_PIPE && !d.compact) {
+            std::vector<int32_t> fc;
+            for (size_t k = 0; k < mask.size(); ++k)
+                if ((mask[k] >> 4) & 1u) fc.push_back((int32_t)k);
+            if (!fc.empty()) LBM_CUDA(c, cudaMemcpy(g + at_pair[m], fc.data(), fc.size() * 4, cudaMemcpyHostToDevice));
+            d.fluidcol = (const int32_t *)(g + at_pair[m]);
         }
         for (int k = 0; k < 2; ++k) {
             const std::vector<int4> &grp = sg[2 * m + k];
@@ -420,6 +430,7 @@ int update_collision(lbm_ctx *c) {
         c->collision = code;
         c->variant = code != 0 ? model_variant(c->precision) : default_variant(c->precision, c->wall);
         c->variant_odd = code != 0 ? model_variant(c->precision) : default_variant_odd(c->precision, c->wall, c->stride);
+        c->shape_set = false;
         drop_graph(c);
     }
     return LBM_OK;
@@ -491,6 +502,8 @@ int build_member(lbm_ctx *c, const lbm_grid *g, const lbm_relax *r, const lbm_fo
         d.scells = ps * g->nz;
     }
     lbm::fastdiv_setup((uint32_t)std::max<int32_t>(d.Ps, 1), d.ps_mul, d.ps_shr);
+    d.Pw = g->geometry == LBM_PIPE && !d.compact ? (int32_t)ncol : d.Ps;
+    lbm::fastdiv_setup((uint32_t)std::max<int32_t>(d.Pw, 1), d.pw_mul, d.pw_shr);
     return LBM_OK;
 }
 
@@ -498,7 +511,17 @@ int build_member(lbm_ctx *c, const lbm_grid *g, const lbm_relax *r, const lbm_fo
 // Launch shape of the step with index t.
 int variant_at(const lbm_ctx *c, int64_t t) { return (t & 1) ? c->variant_odd : c->variant; }
 
-// Whether the even steps of the shapes of several planes per thread run on pairs of cells
+// Below this many stored cells (all members) a step is the latency of one thread's work, which a
+// second cell lengthens: 12 k cells 2.8 us one by one against 3.0 us in pairs, 28 k cells 2.8
+// against 3.0, 110 k cells 5.6 against 4.8 (F32, steps in a row on the GPU).
+constexpr int64_t PAIRS_MIN_CELLS = 60000;
+
+// Whether a step may start while the one before it drains.  Not in FP64: those steps are bound
+// by the FP64 units of each SM, and blocks that arrive early pack onto the SMs the running step
+// leaves free (20 x 20 x 64 pipe: 21 us per step apart, 38 us overlapped).
+bool overlaps(const lbm_ctx *c) { return c->precision != LBM_F64; }
+
+// Whether the steps of the shapes of several planes per thread run on pairs of cells
 // (lbm_pair.cuh): F32 or 16-bit storage, the default model, every member compact and its
 // columns within the pair table's index range.
 bool pairs_of(const lbm_ctx *c) {
@@ -531,9 +554,15 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         a.sg_sel = sk;
     }
     int64_t blk = 0;
-    const bool pairs = zc > 1 && pairs_of(c);
+    const bool pairs = zc > 1 && (c->shape_set || c->stride >= PAIRS_MIN_CELLS) && pairs_of(c);
     a.pairs = pairs;
-    if (zc > 1 && !pairs && c->wall == LBM_BOUZIDI) bs = 128, zc = 1;      // see launch_planes
+    // without pairs one plane per thread is the faster shape (full-way R = 48 pipe, F32: 147.4 us
+    // per step against 149 to 154), also where there are too few cells to give a thread several
+    if (zc > 1 && !pairs && (c->wall == LBM_BOUZIDI || !c->shape_set)) {
+        bs = lbm::SINGLE_THREADS;
+        zc = 1;
+        a.single = 1;
+    }
     for (size_t m = 0; m < c->hm.size(); ++m) {
         const Member &d = c->hm[m];
         a.st[m] = (d.trig && t < d.t_end) ? std::sin(2.0 * M_PI * (double)t / d.period) : 0.0;
@@ -548,7 +577,7 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
                    (lbm::odd_single_planes(d.nz) + lbm::odd_pair_groups(d.nz, lbm::STEP_SHAPES[v].pz));
         } else {
             // threads over (plane group, in-plane position); zc = 1 is every stored cell
-            const int64_t work = (int64_t)d.Ps * ((d.nz + zc - 1) / zc);
+            const int64_t work = (int64_t)d.Pw * ((d.nz + zc - 1) / zc);
             blk += (work + bs - 1) / bs;
         }
     }
@@ -1005,10 +1034,12 @@ int lbm_set_check(lbm_ctx *c, int64_t every, double max_mass_drift) {
 
 namespace {
 
-// One step by a direct launch.
-int step_direct(lbm_ctx *c) {
+// One step by a direct launch.  overlap: the launch before it on the stream is a step of this
+// call, so this one may start while that one drains (timed launches stay apart).
+int step_direct(lbm_ctx *c, bool overlap = false) {
     const bool stats = c->stats && c->stats_every > 0 && (c->t % c->stats_every == 0);
     StepArgs a = make_args(c, c->t);
+    a.overlap = overlap && !c->prof && overlaps(c);
     if (c->skip_tile >= 0 && lbm::staged_of(variant_at(c, c->t)) >= 0) {
         a.skip_tile = c->skip_tile;
         c->skip_tile = -1;
@@ -1063,6 +1094,7 @@ int build_graph(lbm_ctx *c) {
         StepArgs &a = ap[k & 1];
         a.times = c->d_times;
         a.tidx = k;
+        a.overlap = k > 0 && overlaps(c);
         const bool stats = every > 0 && (k % every == 0);
         const int v = variant_at(c, k);
         switch (c->precision) {
@@ -1131,6 +1163,7 @@ extern "C" {
 int lbm_step(lbm_ctx *c, int64_t n) {
     if (!c) return LBM_EINVAL;
     if (n < 0) return set_err(c, LBM_EINVAL, "n must be >= 0");
+    bool overlap = false;
     while (n > 0) {
         const int every = (c->stats && c->stats_every > 0) ? c->stats_every : 0;
         const int64_t t0 = c->t;
@@ -1140,15 +1173,18 @@ int lbm_step(lbm_ctx *c, int64_t n) {
         if (c->graph_chunk > 0 && n >= c->graph_chunk && aligned) {
             rc = step_graph_chunk(c);
             done = c->graph_chunk;
+            overlap = false;
         } else {
-            rc = step_direct(c);
+            rc = step_direct(c, overlap);
             done = 1;
+            overlap = true;
         }
         if (rc) return rc;
         n -= done;
         if (c->check_every > 0 && (c->t / c->check_every) != (t0 / c->check_every)) {
             rc = stability_check(c);
             if (rc) return rc;
+            overlap = false;
         }
     }
     return LBM_OK;
@@ -1204,7 +1240,10 @@ int lbm_set_variants(lbm_ctx *c, int32_t even, int32_t odd) {
     c->variant = even;
     c->variant_odd = odd;
     const int rc = prepare_variant(c);
-    if (rc) {
+    if (rc == LBM_OK) {
+        c->shape_set = true;
+        drop_graph(c);
+    } else {
         c->variant = old_even;
         c->variant_odd = old_odd;
     }
@@ -1256,6 +1295,8 @@ int lbm_autotune(lbm_ctx *c, int32_t steps, int32_t *variant, double *best_us) {
         if (cudaEventCreate(&ev[k]) != cudaSuccess) rc = cuda_err(c, cudaGetLastError(), "autotune events");
     int best[2] = {c->variant, c->variant_odd};
     double best_t[2] = {1e300, 1e300};
+    c->shape_set = true;
+    drop_graph(c);
     for (int v = 0; v < nv && rc == LBM_OK; ++v) {
         if (!variant_available(c, v)) continue;
         c->variant = c->variant_odd = v;
@@ -1564,11 +1605,12 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
         if (sgm < nseg - 1) {
             e = cudaMemcpyAsync((char *)ck + sgm * pop_bytes, c->pops, pop_bytes, cudaMemcpyDeviceToDevice, c->stream);
             if (e != cudaSuccess) { rc = cuda_err(c, e, "checkpoint copy"); break; }
-            for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) rc = step_direct(c);
+            for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) rc = step_direct(c, k > 0);
         } else {
             c->variant = c->variant_odd = lbm::moments_variant(c->precision);
             for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) {
                 StepArgs a = make_args(c, c->t);
+                a.overlap = k > 0 && overlaps(c);
                 a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
                 rc = dispatch(c, [&](auto P) {
                     return lbm::launch_step_moments<decltype(P)::value>((int)(c->t & 1), a, c->stream);
@@ -1621,6 +1663,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
         if (ce != cudaSuccess) return cuda_err(c, ce, "checkpoint restore");
         for (int64_t k = 0; k < ns; ++k) {
             StepArgs a = make_args(c, ts + k);
+            a.overlap = k > 0 && overlaps(c);
             a.pops = work;
             a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
             const int r = dispatch(c, [&](auto P) {
@@ -1641,6 +1684,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
         for (int64_t k = ns - 1; k >= 0 && rc == LBM_OK; --k) {
             const int64_t t = ts + k;
             StepArgs a = make_args(c, t);
+            a.overlap = k < ns - 1 && overlaps(c);
             j.lam_next = (char *)lam + (size_t)((t + 1) & 1) * 27 * n * es;
             j.lam = (char *)lam + (size_t)(t & 1) * 27 * n * es;
             j.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;

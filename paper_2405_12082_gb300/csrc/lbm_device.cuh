@@ -269,6 +269,10 @@ struct Member {
     const void *ztab;          // trigger: [2][nz] cos, sin of kz 2 pi z / L, compute type
     const void *dtab;          // Bouzidi walls: [ny][nx][9][3] coefficients A, B, C of the link
                                // (cx, cy) at index nbit(cx, cy), compute type
+    const int32_t *fluidcol;   // dense pipe: [Pw] dense columns y nx + x of the fluid cells
+    int32_t Pw;                // positions of a plane that threads map to: the fluid columns of a
+                               // dense pipe, else Ps
+    uint32_t pw_mul, pw_shr;   // magic division by Pw
     const uint32_t *pairinfo;  // compact: [Ps / 2] per pair of stored positions (see PAIR_*)
     const void *ftabc;         // trigger, compact: [3][Ps] column factors by stored position
     const int4 *sg[2];         // compact: row groups of the two staged launch shapes (2 int4
@@ -323,7 +327,9 @@ struct StepArgs {
     void *moments;            // adjoint recompute: [9][cells] rho, u, s4..s8 of member 0
     int32_t collision;        // collision model (MODEL_* bits), the same for every member
     uint32_t zero;            // 0 (see store_pops)
-    int32_t pairs;            // an even step on pairs of cells (lbm_pair.cuh)
+    int32_t overlap;          // the kernel may start while the step before it drains
+    int32_t single;           // a shape of several planes per thread runs one (small contexts)
+    int32_t pairs;            // the step runs on pairs of cells (lbm_pair.cuh)
     int32_t stage_cap;        // staged shapes: storage elements per direction segment
     int32_t sg_sel;           // staged shapes: which row-group table (0 or 1)
     int32_t *err;             // device status word (bounded waits that expired), or NULL
@@ -421,6 +427,25 @@ __device__ __forceinline__ bool cell_from_storage(const Member &d, uint32_t sidx
     p.nb = d.colmask[p.y * d.nx + p.x];
     cell_offsets(d, p);
     return (p.nb >> 4) & 1u;
+}
+
+// Cell of thread index `local` of a launch over Pw positions x plane groups of zc planes (the
+// first plane of its group): the fluid columns of a dense pipe are packed, so its warps hold
+// fluid cells only.  Returns whether there is a fluid cell.
+__device__ __forceinline__ bool cell_from_work(const Member &d, uint32_t local, uint32_t zc, CellPos &p) {
+    const uint32_t g = fastdiv(local, d.pw_mul, d.pw_shr);
+    const uint32_t z = g * zc;
+    if (z >= (uint32_t)d.nz) return false;
+    const uint32_t r = local - g * (uint32_t)d.Pw;
+    if (d.fluidcol == nullptr) return cell_from_storage(d, z * (uint32_t)d.Ps + r, p);
+    const uint32_t col = (uint32_t)d.fluidcol[r];
+    p.y = (int)fastdiv(col, d.nx_mul, d.nx_shr);
+    p.x = (int)(col - (uint32_t)p.y * (uint32_t)d.nx);
+    p.z = (int)z;
+    p.lc = p.di = (int32_t)(z * (uint32_t)d.Ps + col);
+    p.nb = d.colmask[col];
+    cell_offsets(d, p);
+    return true;
 }
 
 // Cell of dense index di (< cells).  p.lc is the storage index of a fluid cell (every

@@ -79,6 +79,32 @@ inline void fill_pair_member(PairMember &o, const Member &d) {
     o.omegaf = d.omegaf;
 }
 
+// Programmatic dependent launch.  A step launched with overlap = true may be brought onto the
+// GPU while the step before it drains: it announces its own successor at once, reads its
+// (constant) tables and then waits until every block of the step before it has finished and
+// its writes are visible.  Every step kernel has both calls; without the launch attribute
+// they do nothing.
+__device__ __forceinline__ void release_next_step() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+inline cudaLaunchConfig_t step_config(int blocks, int threads, bool overlap, cudaLaunchAttribute (&at)[1], cudaStream_t s) {
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cfg;
+}
+template <class A>
+cudaError_t launch_step_kernel(void (*kern)(const A), int blocks, int threads, bool overlap, const A &a, cudaStream_t s) {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = step_config(blocks, threads, overlap, at, s);
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
 struct ModesArgs {
     int32_t n_sections, n_rings, n_theta, n_modes;
     double r_over_R[16];
@@ -104,7 +130,11 @@ constexpr StepShape STEP_SHAPES[13] = {{256, 4, 1, 0, 0, 0, 0, 0},    {256, 3, 1
                                        {128, 8, 2, 0, 0, 256, 2, 2},  {128, 8, 4, 0, 0, 128, 4, 4}, {256, 4, 2, 0, 0, 64, 8, 4},
                                        {128, 7, 2, 0, 0, 128, 4, 2},  {128, 6, 2, 0, 0, 128, 4, 8}, {992, 1, 1, 0, 1, 0, 0, 0},
                                        {512, 1, 1, 0, 2, 0, 0, 0}};
-constexpr StepShape STEP_SHAPE_F64 = {256, 2, 1, 0, 0};
+// FP64 steps are bound by the FP64 units of each SM: blocks of one warp spread a small context
+// evenly over the SMs.
+constexpr StepShape STEP_SHAPE_F64 = {32, 16, 1, 0, 0, 0, 0, 0};
+// Threads per block where a shape of several planes per thread runs one (see make_args).
+constexpr int SINGLE_THREADS = 128;
 constexpr int N_STEP_SHAPES = 13;
 // Staged shapes: threads per CTA (one producer warp, the rest consume), pipeline stages
 // (tiles in flight per CTA), CTAs per SM and consumer groups (tiles worked on at once).

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 
 #include "lbm_internal.h"
 #include "lbm_pair.cuh"
@@ -12,7 +13,7 @@
 namespace lbm {
 
 // ---- the fused step: load (stream) + wall + force + MRT collision + store ----------------
-// One thread per cell of every member; solid cells return at once.  EXTRA selects
+// One thread per fluid cell of every member (padding of the compact rows returns at once).  EXTRA selects
 // what else the step does: EX_STATS adds u_z^k, k = 1..4, of the pre-collision state to
 // the FP64 sums (sample steps); EX_MOMENTS stores rho, u and s4..s8 of the
 // pre-collision state for the adjoint sweep.  BS threads per block, register budget
@@ -84,32 +85,22 @@ __device__ __forceinline__ void next_plane(const Member &d, CellPos &p) {
 template <int P, int PAR, int WALL, int EXTRA, int BS, int MINB, int MODEL = MODEL_MRT_H6, int ZC = 1>
 __global__ void __launch_bounds__(BS, MINB) k_step(const __grid_constant__ StepArgs a) {
     using R = typename Storage<P>::R;
+    release_next_step();
     const int m = find_member(a, blockIdx.x);
     const Member &d = a.members[m];
     const uint32_t local = (uint32_t)(blockIdx.x - a.block0[m]) * BS + threadIdx.x;
-    if constexpr (ZC == 1) {
-        if (local >= (uint32_t)d.scells) return;
-        CellPos p;
-        if (!cell_from_storage(d, local, p)) return;
-        const int64_t t = a.times ? a.times[a.tidx].t : a.t;
-        step_cell<P, PAR, WALL, EXTRA, MODEL>(a, d, p, t, st_of<R>(a, m));
-    } else {
-        const uint32_t nzg = (uint32_t)(d.nz + ZC - 1) / ZC;
-        if (local >= (uint32_t)d.Ps * nzg) return;
-        const uint32_t zg = fastdiv(local, d.ps_mul, d.ps_shr);
-        const uint32_t r = local - zg * (uint32_t)d.Ps;
-        CellPos p;
-        if (!cell_from_storage(d, zg * ZC * (uint32_t)d.Ps + r, p)) return;
-        const int64_t t = a.times ? a.times[a.tidx].t : a.t;
-        const R stv = st_of<R>(a, m);
+    CellPos p;
+    if (!cell_from_work(d, local, ZC, p)) return;
+    const int64_t t = a.times ? a.times[a.tidx].t : a.t;
+    const R stv = st_of<R>(a, m);
+    await_previous_step();
 #pragma unroll 1
-        for (int k = 0; k < ZC; ++k) {
-            if (k > 0) {
-                if (p.z + 1 >= d.nz) break;
-                next_plane(d, p);
-            }
-            step_cell<P, PAR, WALL, EXTRA, MODEL>(a, d, p, t, stv);
+    for (int k = 0; k < ZC; ++k) {
+        if (k > 0) {
+            if (p.z + 1 >= d.nz) break;
+            next_plane(d, p);
         }
+        step_cell<P, PAR, WALL, EXTRA, MODEL>(a, d, p, t, stv);
     }
 }
 
@@ -786,6 +777,7 @@ template <int P, int OBJ>
 __global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint(const __grid_constant__ StepArgs a,
                                                                      const AdjArgs j) {
     using R = typename Storage<P>::R;
+    release_next_step();
     const Member &d = a.members[0];
     const uint32_t local = blockIdx.x * 256u + threadIdx.x;
     const uint32_t nzg = (uint32_t)(d.nz + ADJ_ZC - 1) / ADJ_ZC;
@@ -794,7 +786,9 @@ __global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint(const __gri
         const uint32_t zg = fastdiv(local, d.ps_mul, d.ps_shr);
         const uint32_t r = local - zg * (uint32_t)d.Ps;
         CellPos p;
-        if (cell_from_storage(d, zg * ADJ_ZC * (uint32_t)d.Ps + r, p)) {
+        const bool fluid = cell_from_storage(d, zg * ADJ_ZC * (uint32_t)d.Ps + r, p);
+        await_previous_step();
+        if (fluid) {
 #pragma unroll 1
             for (int k = 0; k < ADJ_ZC; ++k) {
                 if (k > 0) {
@@ -816,6 +810,7 @@ __global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint(const __gri
         x1 += __shfl_down_sync(0xFFFFFFFFu, x1, o);
     }
     if ((threadIdx.x & 31) == 0) {
+        await_previous_step();               // (a warp past the last position)
         const int64_t wslot = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
         j.blockacc[wslot] += (double)x0;
         j.blockacc[(int64_t)j.nblocks * 8 + wslot] += (double)x1;
@@ -856,11 +851,12 @@ static inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b -
 
 template <int P, int BS, int MINB, int ZC = 1>
 cudaError_t launch_step_shape(int wall, int parity, bool stats, const StepArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
     LBM_DISPATCH_WP(wall, parity, {
-        if (stats) k_step<P, PA, W, EX_STATS, BS, MINB, MODEL_MRT_H6, ZC><<<a.nblocks_total, BS, 0, s>>>(a);
-        else k_step<P, PA, W, EX_NONE, BS, MINB, MODEL_MRT_H6, ZC><<<a.nblocks_total, BS, 0, s>>>(a);
+        if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
+        else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
     });
-    return cudaGetLastError();
+    return e;
 }
 
 template <int P, int BS, int MINB>
@@ -892,47 +888,59 @@ cudaError_t launch_step_pipe(int wall, int parity, bool stats, const StepArgs &a
 // registers of its shape (half the resident blocks): their populations stay live longer.
 template <int P, int BS, int MINB>
 cudaError_t launch_step_model(int wall, int parity, bool stats, const StepArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
     constexpr int MINB_R = MINB > 1 ? MINB / 2 : 1;
     LBM_DISPATCH_WP(wall, parity, {
         switch (a.collision) {
             case MODEL_BGK:
-                if (stats) k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK><<<a.nblocks_total, BS, 0, s>>>(a);
-                else k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK><<<a.nblocks_total, BS, 0, s>>>(a);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_O2:
-                if (stats) k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
-                else k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_BGK | MODEL_O2:
-                if (stats) k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK | MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
-                else k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK | MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_RATES:
-                if (stats) k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_RATES><<<a.nblocks_total, BS, 0, s>>>(a);
-                else k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_RATES><<<a.nblocks_total, BS, 0, s>>>(a);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_RATES>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_RATES>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_RATES | MODEL_O2:
-                if (stats) k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_RATES | MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
-                else k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_RATES | MODEL_O2><<<a.nblocks_total, BS, 0, s>>>(a);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_RATES | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_RATES | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             default: return cudaErrorInvalidValue;
         }
     });
-    return cudaGetLastError();
+    return e;
 }
 
 // A step of a compact pipe context on pairs of cells, in shape V.
 template <int P, int V, int WALL, class A>
-cudaError_t launch_pair_args(int parity, bool stats, int blocks, const A &a, cudaStream_t s) {
+cudaError_t launch_pair_args(int parity, bool stats, int blocks, bool overlap, const A &a, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
     constexpr StepShape S = STEP_SHAPES[V];
     if (parity == 0) {
-        if (stats) k_even2<P, WALL, EX_STATS, 128, EVEN2_BLOCKS, A><<<blocks, 128, 0, s>>>(a);
-        else k_even2<P, WALL, EX_NONE, 128, EVEN2_BLOCKS, A><<<blocks, 128, 0, s>>>(a);
+        if (stats) e = launch_step_kernel<A>(k_even2<P, WALL, EX_STATS, 128, EVEN2_BLOCKS, A>, blocks, 128, overlap, a, s);
+        else e = launch_step_kernel<A>(k_even2<P, WALL, EX_NONE, 128, EVEN2_BLOCKS, A>, blocks, 128, overlap, a, s);
     } else {
-        if (stats) k_odd2<P, WALL, EX_STATS, S.pt, S.pb, S.pz, A><<<blocks, S.pt, 0, s>>>(a);
-        else k_odd2<P, WALL, EX_NONE, S.pt, S.pb, S.pz, A><<<blocks, S.pt, 0, s>>>(a);
+        if (stats) e = launch_step_kernel<A>(k_odd2<P, WALL, EX_STATS, S.pt, S.pb, S.pz, A>, blocks, S.pt, overlap, a, s);
+        else e = launch_step_kernel<A>(k_odd2<P, WALL, EX_NONE, S.pt, S.pb, S.pz, A>, blocks, S.pt, overlap, a, s);
     }
-    return cudaGetLastError();
+    return e;
+}
+
+// (the lattice functions folded by the compiler: evaluated per launch they took 4 us)
+template <int... I>
+void fill_pull(PairArgsOne &o, uint32_t stride, uint32_t ps, std::integer_sequence<int, I...>) {
+    constexpr int jump[] = {(opp_of(I) - I)...}, cz[] = {cz_of(I)...};
+    for (int i = 0; i < Q; ++i) {
+        o.own[i] = (uint32_t)i * stride;
+        o.pull[i] = (uint32_t)jump[i] * stride - (uint32_t)cz[i] * ps;
+    }
 }
 
 template <int P, int V>
@@ -944,12 +952,9 @@ cudaError_t launch_pair(int wall, int parity, bool stats, const StepArgs &a, con
         o.stf[0] = a.stf[0];
         o.nb_plane = (uint32_t)((hm[0].Ps + STEP_SHAPES[V].pt - 1) / STEP_SHAPES[V].pt);
         fastdiv_setup(o.nb_plane, o.nb_mul, o.nb_shr);
-        for (int i = 0; i < Q; ++i) {
-            o.own[i] = (uint32_t)i * (uint32_t)a.stride;
-            o.pull[i] = (uint32_t)(opp_of(i) - i) * (uint32_t)a.stride - (uint32_t)(cz_of(i) * hm[0].Ps);
-        }
-        return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, o, s)
-                                   : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, o, s);
+        fill_pull(o, (uint32_t)a.stride, (uint32_t)hm[0].Ps, std::make_integer_sequence<int, Q>{});
+        return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, a.overlap, o, s)
+                                   : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, a.overlap, o, s);
     }
     PairArgsMany o;
     fill_pair_args(o, a);
@@ -957,30 +962,30 @@ cudaError_t launch_pair(int wall, int parity, bool stats, const StepArgs &a, con
     o.n_members = a.n_members;
     for (int m = 0; m < a.n_members; ++m) o.stf[m] = a.stf[m];
     for (int m = 0; m <= a.n_members; ++m) o.block0[m] = a.block0[m];
-    return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, o, s)
-                               : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, o, s);
+    return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, a.overlap, o, s)
+                               : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, a.overlap, o, s);
 }
 
-// A shape of several planes per thread: pairs of cells in the compact pipe layouts, else
-// (full-way walls, periodic box) the planes one after the other.
+// A shape of several planes per thread: pairs of cells in the compact pipe layouts, else the
+// planes one after the other, or one plane per thread (make_args decides).
 template <int P, int V>
 cudaError_t launch_planes(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, cudaStream_t s) {
     if (a.pairs) return launch_pair<P, V>(wall, parity, stats, a, hm, s);
     constexpr StepShape S = STEP_SHAPES[V];
-    // (a pipe too wide for the pair tables: its Bouzidi walls run one plane per thread)
-    if (wall == LBM_BOUZIDI) return launch_step_shape<P, 128, 8>(wall, parity, stats, a, s);
+    if (a.single) return launch_step_shape<P, SINGLE_THREADS, 1024 / SINGLE_THREADS>(wall, parity, stats, a, s);
     const bool full = wall == LBM_FULLWAY;
+    cudaError_t e = cudaSuccess;
     auto go = [&](auto pa, auto w) {
         constexpr int PA = decltype(pa)::value, W = decltype(w)::value;
-        if (stats) k_step<P, PA, W, EX_STATS, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc><<<a.nblocks_total, S.threads, 0, s>>>(a);
-        else k_step<P, PA, W, EX_NONE, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc><<<a.nblocks_total, S.threads, 0, s>>>(a);
+        if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc>, a.nblocks_total, S.threads, a.overlap, a, s);
+        else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, S.threads, S.min_blocks, MODEL_MRT_H6, S.zc>, a.nblocks_total, S.threads, a.overlap, a, s);
     };
     using std::integral_constant;
     if (full && parity == 0) go(integral_constant<int, 0>{}, integral_constant<int, LBM_FULLWAY>{});
     else if (full) go(integral_constant<int, 1>{}, integral_constant<int, LBM_FULLWAY>{});
     else if (parity == 0) go(integral_constant<int, 0>{}, integral_constant<int, LBM_HALFWAY>{});
     else go(integral_constant<int, 1>{}, integral_constant<int, LBM_HALFWAY>{});
-    return cudaGetLastError();
+    return e;
 }
 
 template <int P>
@@ -990,12 +995,12 @@ cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, con
     if (a.collision == MODEL_MRT_H6 && STEP_SHAPES[variant].staged)
         return launch_step_staged<P>(wall, parity, stats, a, variant, s);
     if (a.collision != MODEL_MRT_H6) {
-        if constexpr (P == LBM_F64) return launch_step_model<P, 256, 2>(wall, parity, stats, a, s);
+        if constexpr (P == LBM_F64) return launch_step_model<P, STEP_SHAPE_F64.threads, STEP_SHAPE_F64.min_blocks>(wall, parity, stats, a, s);
         else if constexpr (P == LBM_F32) return launch_step_model<P, 128, 8>(wall, parity, stats, a, s);
         else return cudaErrorInvalidValue;
     }
     if constexpr (P == LBM_F64) {
-        return launch_step_shape<P, 256, 2>(wall, parity, stats, a, s);
+        return launch_step_shape<P, STEP_SHAPE_F64.threads, STEP_SHAPE_F64.min_blocks>(wall, parity, stats, a, s);
     } else {
         switch (variant) {
             case 1: return launch_step_shape<P, 256, 3>(wall, parity, stats, a, s);
@@ -1021,11 +1026,11 @@ cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, con
 template <int P>
 cudaError_t launch_step_moments(int parity, const StepArgs &a, cudaStream_t s) {
     if constexpr (P == LBM_F64 || P == LBM_F32) {
-        constexpr int BS = 256, MINB = (P == LBM_F64) ? 2 : 4;
+        constexpr int BS = P == LBM_F64 ? STEP_SHAPE_F64.threads : 256, MINB = P == LBM_F64 ? STEP_SHAPE_F64.min_blocks : 4;
         constexpr int ZC = (P == LBM_F64) ? 1 : STEP_SHAPES[MOM_VARIANT].zc;
-        if (parity == 0) k_step<P, 0, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC><<<a.nblocks_total, BS, 0, s>>>(a);
-        else k_step<P, 1, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC><<<a.nblocks_total, BS, 0, s>>>(a);
-        return cudaGetLastError();
+        if (parity == 0)
+            return launch_step_kernel<StepArgs>(k_step<P, 0, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
+        return launch_step_kernel<StepArgs>(k_step<P, 1, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
     } else {
         return cudaErrorNotSupported;
     }
@@ -1047,9 +1052,10 @@ cudaError_t launch_sum_columns(const double *base, int64_t n, int nv, double *pa
 template <int P>
 cudaError_t launch_adjoint(const StepArgs &a, const AdjArgs &j, cudaStream_t s) {
     if constexpr (P == LBM_F64 || P == LBM_F32) {
-        if (j.objective == LBM_J_UBULK) k_adjoint<P, LBM_J_UBULK><<<j.nblocks, 256, 0, s>>>(a, j);
-        else k_adjoint<P, LBM_J_WSS><<<j.nblocks, 256, 0, s>>>(a, j);
-        return cudaGetLastError();
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg = step_config(j.nblocks, 256, a.overlap, at, s);
+        if (j.objective == LBM_J_UBULK) return cudaLaunchKernelEx(&cfg, k_adjoint<P, LBM_J_UBULK>, a, j);
+        return cudaLaunchKernelEx(&cfg, k_adjoint<P, LBM_J_WSS>, a, j);
     } else {
         return cudaErrorNotSupported;
     }

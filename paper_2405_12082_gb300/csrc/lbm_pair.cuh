@@ -4,7 +4,7 @@
 // Even steps (k_even2): own slots only, so a thread takes two cells that are neighbours in x
 // (an even storage position and the next one: rows start on 64-byte boundaries) and moves
 // each population of the pair with one access of twice the width.  No neighbour data is
-// needed: the 27 loads go out before the position table is read.
+// needed: the 27 loads do not wait for the position table.
 // Odd steps (k_odd2): neighbour slots, which an x pair could only reach with misaligned
 // accesses, so a thread takes the planes z and z + 1 of one position: the same table entry,
 // row offsets, wall links (the wall is a cylinder), link coefficients and, one plane apart,
@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
     using T = typename PS::T;
     using V = typename PS::V;
     constexpr bool SC = P == LBM_F16S;
+    release_next_step();
     const PairTask tk = pair_task(a);
     const auto &d = pair_member(a, tk.m);
     const uint32_t pair = tk.local * BS + threadIdx.x;
@@ -98,14 +99,15 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
     char *const base = static_cast<char *>(a.pops);
     const uint64_t stb = (uint64_t)a.stride * sizeof(T);
     const uint32_t vo = ((uint32_t)d.off + lc) * (uint32_t)sizeof(T);
+    const uint32_t z = fastdiv(lc, d.ps_mul, d.ps_shr);
+    const uint32_t r = lc - z * (uint32_t)d.Ps;
+    const uint32_t pi = d.pairinfo[r >> 1];
+    await_previous_step();
     V raw[Q];
     sfor<0, Q>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         raw[i] = *reinterpret_cast<const V *>(base + i * stb + vo);
     });
-    const uint32_t z = fastdiv(lc, d.ps_mul, d.ps_shr);
-    const uint32_t r = lc - z * (uint32_t)d.Ps;
-    const uint32_t pi = d.pairinfo[r >> 1];
     if (!(pi & PAIR_A)) return;                 // both positions are padding
     const uint32_t col = pi >> PAIR_SHIFT;
     const pf2 act = make_float2(1.f, (pi & PAIR_B) ? 1.f : 0.f);
@@ -311,6 +313,7 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
 // the first blocks take the planes that are left (0, nz - 1 and, for odd nz, nz - 2) singly.
 template <int P, int WALL, int EXTRA, int BS, int MINB, int ZC, class A>
 __global__ void __launch_bounds__(BS, MINB) k_odd2(const __grid_constant__ A a) {
+    release_next_step();
     const PairTask tk = pair_task(a);
     const auto &d = pair_member(a, tk.m);
     uint32_t nb_plane, zg;
@@ -334,6 +337,7 @@ __global__ void __launch_bounds__(BS, MINB) k_odd2(const __grid_constant__ A a) 
         ty = ft[d.Ps];
         tz = ft[2 * (uint32_t)d.Ps];
     }
+    await_previous_step();
     const int singles = odd_single_planes(d.nz);
     if ((int)zg < singles) {
         const int z = zg == 0 ? 0 : d.nz - (int)zg;
