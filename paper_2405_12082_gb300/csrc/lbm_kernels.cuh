@@ -431,6 +431,21 @@ __device__ __forceinline__ void block_sum(double (&x)[NV], double *sh /* [NV][32
     }
 }
 
+// FP64 adds are what a sum of FP32 populations costs here (two lanes per SM and cycle: 81 adds
+// and 27 conversions per cell took 10 ms on the R = 96 pipe, against 0.55 ms for reading it).
+// So every thread keeps each population's sum over eight cells as an unevaluated pair hi + lo of
+// floats -- Knuth's two-sum: hi + x = s + e exactly, e collected in lo, about 48 bits -- and
+// only the pairs of eight cells enter FP64, through the z-triplets of moment_sums: 17 FP64
+// operations per cell.  A pair's rounding stays below that of the FP64 sum of a thread's
+// hundred cells it joins.  Cells with a value too large for FP32 sums (or not finite) are
+// added in FP64 one by one.
+constexpr int REDUCE_CELLS = 8;
+__device__ __forceinline__ void add_sums(double (&acc)[5], const MomentSums<double> &m) {
+    acc[0] += m.drho;
+    acc[1] += m.jx;
+    acc[2] += m.jy;
+    acc[3] += m.jz;
+}
 template <int P, int PAR, int WALL>
 __global__ void __launch_bounds__(REDUCE_BLOCK) k_reduce(const __grid_constant__ StepArgs a, int m,
                                                          double *partials) {
@@ -438,29 +453,51 @@ __global__ void __launch_bounds__(REDUCE_BLOCK) k_reduce(const __grid_constant__
     __shared__ double sh[5 * 32];
     const Member &d = a.members[m];
     double acc[5] = {0, 0, 0, 0, 0};
-    for (int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; local < d.cells;
+    float hi[Q], lo[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) hi[i] = lo[i] = 0.f;
+    int held = 0;
+    auto flush = [&]() {
+        double x[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            x[i] = __dadd_rn((double)hi[i], (double)lo[i]);
+            hi[i] = lo[i] = 0.f;
+        }
+        add_sums(acc, moment_sums<double>(x));
+        held = 0;
+    };
+    const int64_t work = (int64_t)d.Pw * d.nz;
+    for (int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; local < work;
          local += (int64_t)gridDim.x * blockDim.x) {
         CellPos p;
-        if (!cell_from_dense(d, (uint32_t)local, p)) continue;
+        if (!cell_from_work(d, (uint32_t)local, 1, p)) continue;
         R v[Q];
         load_pops<P, PAR, WALL>(a, d, p, v);
-        double dr = 0, jx = 0, jy = 0, jz = 0;
-        bool bad = false;
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            const double x = (double)v[i];
-            bad |= !isfinite(x);
-            dr += x;
-            jx += cx_of(i) * x;
-            jy += cy_of(i) * x;
-            jz += cz_of(i) * x;
-        });
-        acc[0] += dr;
-        acc[1] += jx;
-        acc[2] += jy;
-        acc[3] += jz;
-        acc[4] += bad ? 1.0 : 0.0;
+        bool wide = false;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) wide |= !(fabs(v[i]) < R(1e30));
+        if (sizeof(R) == 8 || wide) {
+            double x[Q];
+            bool bad = false;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                x[i] = (double)v[i];
+                bad |= !isfinite(x[i]);
+            }
+            add_sums(acc, moment_sums<double>(x));
+            acc[4] += bad ? 1.0 : 0.0;
+        } else if constexpr (sizeof(R) == 4) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const float s = __fadd_rn(hi[i], v[i]), t = __fsub_rn(s, hi[i]);
+                lo[i] = __fadd_rn(lo[i], __fadd_rn(__fsub_rn(hi[i], __fsub_rn(s, t)), __fsub_rn(v[i], t)));
+                hi[i] = s;
+            }
+            if (++held == REDUCE_CELLS) flush();
+        }
     }
+    if (held > 0) flush();
     block_sum<5>(acc, sh);
     if (threadIdx.x == 0)
 #pragma unroll
@@ -494,19 +531,27 @@ __device__ double uz_at(const StepArgs &a, const Member &d, int m, int x, int y,
 }
 
 // One block per (section, ring): bilinear samples of u_z into shared memory, then the
-// DFT energies E_m = |sum_n u_n e^{-i m theta_n}|^2 / N^2 with warp-shuffle sums.
+// DFT energies E_m = |sum_n u_n e^{-i m theta_n}|^2 / N^2 with warp-shuffle sums.  The N
+// angles' sines and cosines (FP64: the slow units of this chip) are taken once per block, for
+// the sample positions, and serve the DFT as its table: m n mod N, stepped without a division.
+// 3 rings x 16 sections of 1024 samples, m to 32, R = 96 pipe: 1.9 ms -> 0.1 ms.
+constexpr int MODES_BLOCK = 512;
 template <int P, int PAR, int WALL>
-__global__ void k_modes(const __grid_constant__ StepArgs a, int m, const ModesArgs ma, double *E) {
-    extern __shared__ double smp[];
+__global__ void __launch_bounds__(MODES_BLOCK) k_modes(const __grid_constant__ StepArgs a, int m, const ModesArgs ma,
+                                                       double *E) {
+    extern __shared__ double smp[];            // [3][N]: u_z, cos, sin
     const Member &d = a.members[m];
     const int s = blockIdx.x / ma.n_rings, j = blockIdx.x % ma.n_rings;
     const int z = (int)(((int64_t)s * d.nz) / ma.n_sections);
     const int N = ma.n_theta;
+    double *const cosn = smp + N, *const sinn = smp + 2 * N;
     const double xc = 0.5 * (d.nx - 1), yc = 0.5 * (d.ny - 1);
     const double r = ma.r_over_R[j] * d.R;
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
         double sn, cs;
         sincospi(2.0 * (double)n / (double)N, &sn, &cs);
+        cosn[n] = cs;
+        sinn[n] = sn;
         const double px = xc + r * cs, py = yc + r * sn;
         const int i0 = (int)floor(px), j0 = (int)floor(py);
         const double fx = px - i0, fy = py - j0;
@@ -520,12 +565,13 @@ __global__ void k_modes(const __grid_constant__ StepArgs a, int m, const ModesAr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int mode = warp; mode <= ma.n_modes; mode += nw) {
         double re = 0, im = 0;
+        const int step = (int)(((int64_t)mode * 32) % N);
+        int k = (int)(((int64_t)mode * lane) % N);          // mode n mod N
         for (int n = lane; n < N; n += 32) {
-            const int64_t k = ((int64_t)mode * n) % N;
-            double sn, cs;
-            sincospi(2.0 * (double)k / (double)N, &sn, &cs);
-            re += smp[n] * cs;
-            im -= smp[n] * sn;
+            re += smp[n] * cosn[k];
+            im -= smp[n] * sinn[k];
+            k += step;
+            if (k >= N) k -= N;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1137,13 +1183,13 @@ cudaError_t launch_modes(int wall, int parity, const StepArgs &a, const Member &
                          double *E, cudaStream_t s) {
     (void)hm;
     const int nblk = ma.n_sections * ma.n_rings;
-    const size_t shm = (size_t)ma.n_theta * sizeof(double);
+    const size_t shm = 3 * (size_t)ma.n_theta * sizeof(double);
     LBM_DISPATCH_WP(wall, parity, {
         if (shm > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_modes<P, PA, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
             if (e != cudaSuccess) return e;
         }
-        k_modes<P, PA, W><<<nblk, 256, shm, s>>>(a, m, ma, E);
+        k_modes<P, PA, W><<<nblk, MODES_BLOCK, shm, s>>>(a, m, ma, E);
     });
     return cudaGetLastError();
 }
