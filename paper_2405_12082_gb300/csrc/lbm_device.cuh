@@ -820,12 +820,20 @@ template <int E, class R> __device__ __forceinline__ R cterm(R acc, R x) {
 // ACT: the outputs are multiplied by act (1, or 0 for the padding half of a pair, which must
 // stay zero) through the four factors they all carry.
 // LEAN (see macro_from_sums): X = G (1 + dz) + hz D + (dz + hz), 15 operations fewer.
-template <class R, bool SCALED, bool ACT, bool LEAN, class Emit>
+//
+// MODEL_BGK: f* = f + omega (f^eq - f) + (2 - omega) F/2 = f + omega (w drho + w rho X - (f - w))
+// with h scaled by (2 - omega) / omega in X; the populations f - w are read from fin.  (Folding
+// omega into the weights saves an operation per population and rounds the momentum of all
+// of them alike once more: 1.05e-5 instead of 5e-6 off after 1,000 laminar steps.)
+// MODEL_O2: X = 9/2 (c.u)(c.w) + 3/2 (c.u + c.w) - 3/2 u.w with w = u + g (that factor times g
+// for the BGK), evaluated for c and -c together: even part plus and minus odd part.
+template <class R, bool SCALED, bool ACT, bool LEAN, int MODEL = 0, class Emit>
 __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R gy, R gz,
                                                 typename scalar_of<R>::type omega, typename scalar_of<R>::type inv,
                                                 typename scalar_of<R>::type sc, R *s_out, Emit &&emit,
-                                                R act = lit<R>(1)) {
+                                                R act = lit<R>(1), const R *fin = nullptr) {
     using S = typename scalar_of<R>::type;
+    constexpr bool bgk = (MODEL & MODEL_BGK) != 0, o2 = (MODEL & MODEL_O2) != 0;
     const R hgx = mul_(lit<R>(0.5f), gx), hgy = mul_(lit<R>(0.5f), gy), hgz = mul_(lit<R>(0.5f), gz);
     const Macro<R> mm = macro_from_sums<R, SCALED, LEAN>(ms, hgx, hgy, hgz, inv);
     const R rho = mm.rho;
@@ -853,9 +861,83 @@ __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R
         rho_o = mul_(rho_o, act);
         drho_o = mul_(drho_o, act);
     }
-    const R b7 = mul_(om6, s7), b8 = mul_(om6, s8);
-    const R s12 = fma_(om6, s7, b8), s34 = fma_(lit<R>(-2), b7, b8), s56 = fma_(lit<R>(-2), b8, b7);
-    const R q4 = mul_(om4, s4), q5 = mul_(om4, s5), q6 = mul_(om4, s6);
+    R s12 = lit<R>(0), s34 = s12, s56 = s12, q4 = s12, q5 = s12, q6 = s12;
+    R kx = hgx, ky = hgy, kz = hgz;             // half the force that enters X
+    if constexpr (bgk) {
+        const R kap = lit<R>((S(2) - omega) * recip_(omega));
+        kx = mul_(kap, hgx);
+        ky = mul_(kap, hgy);
+        kz = mul_(kap, hgz);
+    } else {
+        const R b7 = mul_(om6, s7), b8 = mul_(om6, s8);
+        s12 = fma_(om6, s7, b8);
+        s34 = fma_(lit<R>(-2), b7, b8);
+        s56 = fma_(lit<R>(-2), b8, b7);
+        q4 = mul_(om4, s4);
+        q5 = mul_(om4, s5);
+        q6 = mul_(om4, s6);
+    }
+    // w rho and w drho (plus the shear term of the population) per weight shell
+    const S f = SCALED ? sc : S(1);
+    const R wr0 = mul_(lit<R>(S(w_of(0)) * f), rho_o), wr1 = mul_(lit<R>(S(w_of(1)) * f), rho_o);
+    const R wr2 = mul_(lit<R>(S(w_of(7)) * f), rho_o), wr3 = mul_(lit<R>(S(w_of(19)) * f), rho_o);
+    const R w1 = lit<R>(S(w_of(1))), w2 = lit<R>(S(w_of(7)));
+    const R wd0 = mul_(lit<R>(S(w_of(0))), drho_o), wd3 = mul_(lit<R>(S(w_of(19))), drho_o);
+    const R c12 = fma_(w1, drho_o, s12), c34 = fma_(w1, drho_o, s34), c56 = fma_(w1, drho_o, s56);
+    const R c4p = fma_(w2, drho_o, q4), c4m = fma_(w2, drho_o, neg_(q4)), c5p = fma_(w2, drho_o, q5);
+    const R c5m = fma_(w2, drho_o, neg_(q5)), c6p = fma_(w2, drho_o, q6), c6m = fma_(w2, drho_o, neg_(q6));
+    auto put = [&](auto ic, R X) {
+        constexpr int i = decltype(ic)::value;
+        R wr, wd;
+        if constexpr (i == 0) { wr = wr0; wd = wd0; }
+        else if constexpr (i <= 6) {
+            wr = wr1;
+            wd = (i <= 2) ? c12 : ((i <= 4) ? c34 : c56);
+        } else if constexpr (i <= 18) {
+            wr = wr2;
+            if constexpr (i == 7 || i == 10) wd = c4p;
+            else if constexpr (i == 8 || i == 9) wd = c4m;
+            else if constexpr (i == 11 || i == 14) wd = c5p;
+            else if constexpr (i == 12 || i == 13) wd = c5m;
+            else if constexpr (i == 15 || i == 18) wd = c6p;
+            else wd = c6m;
+        } else { wr = wr3; wd = wd3; }
+        if constexpr (bgk) emit(ic, fma_(lit<R>(omega), sub_(fma_(wr, X, wd), fin[i]), fin[i]));
+        else emit(ic, fma_(wr, X, wd));
+    };
+    if constexpr (o2) {
+        const R wx = fma_(lit<R>(2), kx, mm.ux), wy = fma_(lit<R>(2), ky, mm.uy), wz = fma_(lit<R>(2), kz, mm.uz);
+        const R ne0 = mul_(lit<R>(-1.5f), fma_(mm.ux, wx, fma_(mm.uy, wy, mul_(mm.uz, wz))));
+        put(std::integral_constant<int, 0>{}, ne0);
+        sfor<1, Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value, ib = opp_of(i);
+            if constexpr (i < ib) {
+                auto dot = [](R x, R y, R z) {
+                    constexpr int ex = cx_of(i), ey = cy_of(i), ez = cz_of(i);
+                    auto term = [](auto e, R acc, R q) {
+                        constexpr int k = decltype(e)::value;
+                        if constexpr (k == 1) return add_(acc, q);
+                        else if constexpr (k == -1) return sub_(acc, q);
+                        else return acc;
+                    };
+                    using std::integral_constant;
+                    if constexpr (ex != 0) {
+                        const R t = ex > 0 ? x : neg_(x);
+                        return term(integral_constant<int, ez>{}, term(integral_constant<int, ey>{}, t, y), z);
+                    } else if constexpr (ey != 0) {
+                        return term(integral_constant<int, ez>{}, ey > 0 ? y : neg_(y), z);
+                    } else {
+                        return ez > 0 ? z : neg_(z);
+                    }
+                };
+                const R cu = dot(mm.ux, mm.uy, mm.uz), cw = dot(wx, wy, wz);
+                const R even = fma_(mul_(lit<R>(4.5f), cu), cw, ne0), odd = add_(cu, cw);
+                put(ic, fma_(lit<R>(1.5f), odd, even));
+                put(std::integral_constant<int, ib>{}, fma_(lit<R>(-1.5f), odd, even));
+            }
+        });
+        return mm;
+    }
     // one-axis factors at c = -1, 0, +1: d, h and p = 1 + d (those of x row by row).  No sum
     // takes a product that is rounded by itself: the compiler fuses those on pairs and not on
     // single cells, and the two would differ in the last bit.
@@ -875,24 +957,15 @@ __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R
     R dy[3], hy[3], py[3], dz[3], hz[3], pz[3], ez[3];
     sfor<0, 3>([&](auto cc) {
         constexpr int c = decltype(cc)::value;
-        axis(cc, mm.uy, hgy, dy[c], hy[c], py[c]);
-        axis(cc, mm.uz, hgz, dz[c], hz[c], pz[c]);
+        axis(cc, mm.uy, ky, dy[c], hy[c], py[c]);
+        axis(cc, mm.uz, kz, dz[c], hz[c], pz[c]);
         if constexpr (c == 1) ez[c] = fma_(lit<R>(-1.5f), mul_(mm.uz, mm.uz), hz[c]);
         else ez[c] = add_(dz[c], hz[c]);
     });
-    // w rho and w drho (plus the shear term of the population) per weight shell
-    const S f = SCALED ? sc : S(1);
-    const R wr0 = mul_(lit<R>(S(w_of(0)) * f), rho_o), wr1 = mul_(lit<R>(S(w_of(1)) * f), rho_o);
-    const R wr2 = mul_(lit<R>(S(w_of(7)) * f), rho_o), wr3 = mul_(lit<R>(S(w_of(19)) * f), rho_o);
-    const R w1 = lit<R>(S(w_of(1))), w2 = lit<R>(S(w_of(7)));
-    const R wd0 = mul_(lit<R>(S(w_of(0))), drho_o), wd3 = mul_(lit<R>(S(w_of(19))), drho_o);
-    const R c12 = fma_(w1, drho_o, s12), c34 = fma_(w1, drho_o, s34), c56 = fma_(w1, drho_o, s56);
-    const R c4p = fma_(w2, drho_o, q4), c4m = fma_(w2, drho_o, neg_(q4)), c5p = fma_(w2, drho_o, q5);
-    const R c5m = fma_(w2, drho_o, neg_(q5)), c6p = fma_(w2, drho_o, q6), c6m = fma_(w2, drho_o, neg_(q6));
     sfor<0, 3>([&](auto ac) {
         constexpr int a = decltype(ac)::value;
         R dx, hx, px;
-        axis(ac, mm.ux, hgx, dx, hx, px);
+        axis(ac, mm.ux, kx, dx, hx, px);
         sfor<0, 3>([&](auto bc) {
             constexpr int b = decltype(bc)::value;
             const R D = fma_(dy[b], px, dx);
@@ -903,21 +976,7 @@ __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R
                 R X;
                 if constexpr (LEAN) X = fma_(G, pz[c], fma_(hz[c], D, ez[c]));
                 else X = fma_(dz[c], H, fma_(hz[c], A, G));
-                R wr, wd;
-                if constexpr (i == 0) { wr = wr0; wd = wd0; }
-                else if constexpr (i <= 6) {
-                    wr = wr1;
-                    wd = (i <= 2) ? c12 : ((i <= 4) ? c34 : c56);
-                } else if constexpr (i <= 18) {
-                    wr = wr2;
-                    if constexpr (i == 7 || i == 10) wd = c4p;
-                    else if constexpr (i == 8 || i == 9) wd = c4m;
-                    else if constexpr (i == 11 || i == 14) wd = c5p;
-                    else if constexpr (i == 12 || i == 13) wd = c5m;
-                    else if constexpr (i == 15 || i == 18) wd = c6p;
-                    else wd = c6m;
-                } else { wr = wr3; wd = wd3; }
-                emit(std::integral_constant<int, i>{}, fma_(wr, X, wd));
+                put(std::integral_constant<int, i>{}, X);
             });
         });
     });
@@ -940,62 +999,28 @@ __device__ __forceinline__ Macro<R> collide(R (&v)[Q], R gx, R gy, R gz, R omega
                                             const R *lam1 = nullptr, R inv = R(1), R sc = R(1)) {
     static_assert(!SCALED || MODEL == MODEL_MRT_H6, "scaled units serve the default model only");
     const MomentSums<R> ms = moment_sums<R>(v);
-    if constexpr (MODEL == MODEL_MRT_H6) {
-        return collide_mrt<R, SCALED, false, LEAN>(ms, gx, gy, gz, omega, inv, sc, s_out,
-                                      [&](auto ic, R f) { v[decltype(ic)::value] = f; });
+    if constexpr (!(MODEL & MODEL_RATES)) {
+        return collide_mrt<R, SCALED, false, LEAN, MODEL>(ms, gx, gy, gz, omega, inv, sc, s_out,
+                                                          [&](auto ic, R f) { v[decltype(ic)::value] = f; }, R(1), v);
     } else {
-        constexpr bool rates = (MODEL & MODEL_RATES) != 0;
-        constexpr bool bgk = !rates && (MODEL & MODEL_BGK) != 0, o2 = (MODEL & MODEL_O2) != 0;
+        constexpr bool o2 = (MODEL & MODEL_O2) != 0;
         const Macro<R> mm = macro_from_sums<R>(ms, R(0.5) * gx, R(0.5) * gy, R(0.5) * gz);
         const R rho = mm.rho, ux = mm.ux, uy = mm.uy, uz = mm.uz, drho = ms.drho;
-        const R om1 = R(1) - omega;
-        R s12 = 0, s34 = 0, s56 = 0, q4 = 0, q5 = 0, q6 = 0;
-        R mk[23];                 // MODEL_RATES: moments 4..26 of n
+        R mk[23];                 // moments 4..26 of n = f - f^eq + F/2
 #pragma unroll
         for (int k = 0; k < 23; ++k) mk[k] = 0;
-        if constexpr (!bgk && !rates) {
-            // (1 - omega)(m_k - m_k^eq + R_k / 2), k = 4..8, with the printed m^eq and R
-            const R a4 = om1 * (ms.m4 - rho * ux * uy + R(0.5) * rho * (gy * ux + gx * uy));
-            const R a5 = om1 * (ms.m5 - rho * ux * uz + R(0.5) * rho * (gz * ux + gx * uz));
-            const R a6 = om1 * (ms.m6 - rho * uy * uz + R(0.5) * rho * (gz * uy + gy * uz));
-            const R a7 = om1 * (ms.m7 - rho * (ux * ux - uy * uy) + rho * (gx * ux - gy * uy));
-            const R a8 = om1 * (ms.m8 - rho * (ux * ux - uz * uz) + rho * (gx * ux - gz * uz));
-            s12 = (a7 + a8) * R(1.0 / 6.0);
-            s34 = a8 * R(1.0 / 6.0) - a7 * R(1.0 / 3.0);
-            s56 = a7 * R(1.0 / 6.0) - a8 * R(1.0 / 3.0);
-            q4 = R(0.25) * a4;
-            q5 = R(0.25) * a5;
-            q6 = R(0.25) * a6;
-        }
-        // post-collision value of population i from the equilibrium part pm1 = f^eq / (w rho) - 1
-        // and frc = (1/2) g . grad_u (f^eq / (w rho))
+        // v_i becomes f^eq + F/2, from the equilibrium part pm1 = f^eq / (w rho) - 1 and
+        // frc = (1/2) g . grad_u (f^eq / (w rho))
         auto emit = [&](auto ic, R pm1, R frc) {
             constexpr int i = decltype(ic)::value;
-            if constexpr (rates) {
-                const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
-                const R ni = v[i] - eq + fh;
-                sfor<4, Q>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    constexpr int cik = mt_coef(k, i);
-                    if constexpr (cik != 0) mk[k - 4] += R(cik) * ni;
-                });
-                v[i] = eq + fh;
-            } else if constexpr (bgk) {
-                const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
-                v[i] = eq + fh + om1 * (v[i] - eq + fh);
-            } else {
-                R f = R(w_of(i)) * (drho + rho * (pm1 + frc));
-                if constexpr (i == 1 || i == 2) f += s12;
-                if constexpr (i == 3 || i == 4) f += s34;
-                if constexpr (i == 5 || i == 6) f += s56;
-                if constexpr (i == 7 || i == 10) f += q4;
-                if constexpr (i == 8 || i == 9) f -= q4;
-                if constexpr (i == 11 || i == 14) f += q5;
-                if constexpr (i == 12 || i == 13) f -= q5;
-                if constexpr (i == 15 || i == 18) f += q6;
-                if constexpr (i == 16 || i == 17) f -= q6;
-                v[i] = f;
-            }
+            const R eq = R(w_of(i)) * (drho + rho * pm1), fh = R(w_of(i)) * rho * frc;
+            const R ni = v[i] - eq + fh;
+            sfor<4, Q>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                constexpr int cik = mt_coef(k, i);
+                if constexpr (cik != 0) mk[k - 4] += R(cik) * ni;
+            });
+            v[i] = eq + fh;
         };
         if constexpr (!o2) {
             R dx[3], hx[3], dy[3], hy[3], dz[3], hz[3];
@@ -1034,20 +1059,18 @@ __device__ __forceinline__ Macro<R> collide(R (&v)[Q], R gx, R gy, R gz, R omega
                 emit(ic, pm1, frc);
             });
         }
-        if constexpr (rates) {
 #pragma unroll
-            for (int k = 0; k < 23; ++k) mk[k] *= lam1[k];
-            sfor<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                R acc = v[i];
-                sfor<4, Q>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    constexpr double aik = kMtInv.a[i][k];
-                    if constexpr (aik != 0.0) acc += R(aik) * mk[k - 4];
-                });
-                v[i] = acc;
+        for (int k = 0; k < 23; ++k) mk[k] *= lam1[k];
+        sfor<0, Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            R acc = v[i];
+            sfor<4, Q>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                constexpr double aik = kMtInv.a[i][k];
+                if constexpr (aik != 0.0) acc += R(aik) * mk[k - 4];
             });
-        }
+            v[i] = acc;
+        });
         return mm;
     }
 }

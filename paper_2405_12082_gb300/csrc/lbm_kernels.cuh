@@ -930,25 +930,28 @@ cudaError_t launch_step_pipe(int wall, int parity, bool stats, const StepArgs &a
     return cudaGetLastError();
 }
 
-// The ablation models run in the default thread count of the precision with twice the
-// registers of its shape (half the resident blocks): their populations stay live longer.
+// The ablation models run in the thread count of shape 2.  The BGK and the second-order
+// equilibrium fit its 64 registers on even and 72 on odd steps (128 before, when each
+// population went through its own equilibrium); FP64, and general rates, which hold 27
+// populations and 23 moments, take half the resident blocks.
 template <int P, int BS, int MINB>
 cudaError_t launch_step_model(int wall, int parity, bool stats, const StepArgs &a, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     constexpr int MINB_R = MINB > 1 ? MINB / 2 : 1;
     LBM_DISPATCH_WP(wall, parity, {
+        constexpr int MINB_C = P == LBM_F64 ? MINB_R : MINB - PA;
         switch (a.collision) {
             case MODEL_BGK:
-                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
-                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_C, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_C, MODEL_BGK>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_O2:
-                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
-                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_C, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_C, MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_BGK | MODEL_O2:
-                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
-                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_R, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_C, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
+                else e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_NONE, BS, MINB_C, MODEL_BGK | MODEL_O2>, a.nblocks_total, BS, a.overlap, a, s);
                 break;
             case MODEL_RATES:
                 if (stats) e = launch_step_kernel<StepArgs>(k_step<P, PA, W, EX_STATS, BS, MINB_R, MODEL_RATES>, a.nblocks_total, BS, a.overlap, a, s);
