@@ -447,7 +447,7 @@ __device__ __forceinline__ void add_sums(double (&acc)[5], const MomentSums<doub
     acc[3] += m.jz;
 }
 template <int P, int PAR, int WALL>
-__global__ void __launch_bounds__(REDUCE_BLOCK) k_reduce(const __grid_constant__ StepArgs a, int m,
+__global__ void __launch_bounds__(REDUCE_BLOCK, 2) k_reduce(const __grid_constant__ StepArgs a, int m,
                                                          double *partials) {
     using R = typename Storage<P>::R;
     __shared__ double sh[5 * 32];
@@ -456,7 +456,6 @@ __global__ void __launch_bounds__(REDUCE_BLOCK) k_reduce(const __grid_constant__
     float hi[Q], lo[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) hi[i] = lo[i] = 0.f;
-    int held = 0;
     auto flush = [&]() {
         double x[Q];
 #pragma unroll
@@ -465,39 +464,43 @@ __global__ void __launch_bounds__(REDUCE_BLOCK) k_reduce(const __grid_constant__
             hi[i] = lo[i] = 0.f;
         }
         add_sums(acc, moment_sums<double>(x));
-        held = 0;
     };
     const int64_t work = (int64_t)d.Pw * d.nz;
+    int held = 0;                          // counted per pass, not per cell: all lanes flush together
     for (int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; local < work;
          local += (int64_t)gridDim.x * blockDim.x) {
         CellPos p;
-        if (!cell_from_work(d, (uint32_t)local, 1, p)) continue;
-        R v[Q];
-        load_pops<P, PAR, WALL>(a, d, p, v);
-        bool wide = false;
+        if (cell_from_work(d, (uint32_t)local, 1, p)) {
+            R v[Q];
+            load_pops<P, PAR, WALL>(a, d, p, v);
+            bool wide = false;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) wide |= !(fabs(v[i]) < R(1e30));
-        if (sizeof(R) == 8 || wide) {
-            double x[Q];
-            bool bad = false;
+            for (int i = 0; i < Q; ++i) wide |= !(fabs(v[i]) < R(1e30));
+            if (sizeof(R) == 8 || wide) {
+                double x[Q];
+                bool bad = false;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                x[i] = (double)v[i];
-                bad |= !isfinite(x[i]);
+                for (int i = 0; i < Q; ++i) {
+                    x[i] = (double)v[i];
+                    bad |= !isfinite(x[i]);
+                }
+                add_sums(acc, moment_sums<double>(x));
+                acc[4] += bad ? 1.0 : 0.0;
+            } else if constexpr (sizeof(R) == 4) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const float s = __fadd_rn(hi[i], v[i]), t = __fsub_rn(s, hi[i]);
+                    lo[i] = __fadd_rn(lo[i], __fadd_rn(__fsub_rn(hi[i], __fsub_rn(s, t)), __fsub_rn(v[i], t)));
+                    hi[i] = s;
+                }
             }
-            add_sums(acc, moment_sums<double>(x));
-            acc[4] += bad ? 1.0 : 0.0;
-        } else if constexpr (sizeof(R) == 4) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const float s = __fadd_rn(hi[i], v[i]), t = __fsub_rn(s, hi[i]);
-                lo[i] = __fadd_rn(lo[i], __fadd_rn(__fsub_rn(hi[i], __fsub_rn(s, t)), __fsub_rn(v[i], t)));
-                hi[i] = s;
-            }
-            if (++held == REDUCE_CELLS) flush();
+        }
+        if (sizeof(R) == 4 && ++held == REDUCE_CELLS) {
+            flush();
+            held = 0;
         }
     }
-    if (held > 0) flush();
+    if (sizeof(R) == 4) flush();
     block_sum<5>(acc, sh);
     if (threadIdx.x == 0)
 #pragma unroll
