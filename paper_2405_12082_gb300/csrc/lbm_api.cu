@@ -1573,9 +1573,11 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
     if (e == cudaSuccess) e = dev_alloc(c, &mom, mom_seg * (nseg > 1 ? 2 : 1));
     if (e == cudaSuccess) e = dev_alloc(c, &lam, 2 * 27 * n * es);
     if (e == cudaSuccess) e = dev_alloc(c, &accseg, n * es);
-    // adjoint kernel: 256 threads over (plane pair, stored position)
-    const int64_t nblk = ((int64_t)d.Ps * ((d.nz + lbm::ADJ_ZC - 1) / lbm::ADJ_ZC) + 255) / 256;
-    const int64_t nslot = nblk * 8;                  // one slot per warp
+    lbm::AdjArgs j;
+    std::memset(&j, 0, sizeof j);
+    if (c->precision == LBM_F64) lbm::prepare_adjoint<LBM_F64>(j, d);
+    else lbm::prepare_adjoint<LBM_F32>(j, d);
+    const int64_t nslot = (int64_t)j.nblocks * (lbm::ADJ_THREADS / 32);     // one slot per warp
     if (e == cudaSuccess) e = dev_alloc(c, (void **)&acc, (nd + 2 * nslot) * sizeof(double));
     auto release = [&]() {
         dev_free(c, ck); dev_free(c, work); dev_free(c, mom); dev_free(c, lam); dev_free(c, acc); dev_free(c, accseg);
@@ -1599,7 +1601,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
     const int64_t t0 = c->t;
     // forward pass: a checkpoint at the start of every segment but the last, whose steps
     // store their moments at once (its recompute is skipped in the reverse sweep); the
-    // moment-storing kernel runs in the shape moments_variant
+    // moment-storing kernel runs in a shape of its own
     for (int64_t sgm = 0; sgm < nseg && rc == LBM_OK; ++sgm) {
         const int64_t ns = std::min<int64_t>(K, T - sgm * K);
         if (sgm < nseg - 1) {
@@ -1607,13 +1609,13 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
             if (e != cudaSuccess) { rc = cuda_err(c, e, "checkpoint copy"); break; }
             for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) rc = step_direct(c, k > 0);
         } else {
-            c->variant = c->variant_odd = lbm::moments_variant(c->precision);
+            c->variant = c->variant_odd = c->stride >= PAIRS_MIN_CELLS && pairs_of(c) ? lbm::MOM_VARIANT_PAIRS : lbm::MOM_VARIANT;
             for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) {
                 StepArgs a = make_args(c, c->t);
                 a.overlap = k > 0 && overlaps(c);
                 a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
                 rc = dispatch(c, [&](auto P) {
-                    return lbm::launch_step_moments<decltype(P)::value>((int)(c->t & 1), a, c->stream);
+                    return lbm::launch_step_moments<decltype(P)::value>((int)(c->t & 1), a, c->hm.data(), c->stream);
                 });
                 c->t++;
             }
@@ -1621,8 +1623,6 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
     }
     const int64_t t_end = c->t;
     int64_t nfl = d.n_fluid;
-    lbm::AdjArgs j;
-    std::memset(&j, 0, sizeof j);
     j.objective = objective;
     j.kappa = 1.0 / ((double)T * (double)std::max<int64_t>(nfl, 1));
     j.wss = 2.0 / ((double)T * 2.0 * M_PI * d.R * (double)d.nz);
@@ -1631,7 +1631,6 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
     j.acc = acc;
     j.acc_seg = accseg;
     j.blockacc = acc + nd;
-    j.nblocks = (int32_t)nblk;
     if (rc == LBM_OK) {
         e = cudaMemsetAsync(lam, 0, 2 * 27 * n * es, c->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, (nd + 2 * nslot) * sizeof(double), c->stream);
@@ -1667,7 +1666,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
             a.pops = work;
             a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
             const int r = dispatch(c, [&](auto P) {
-                return lbm::launch_step_moments<decltype(P)::value>((int)((ts + k) & 1), a, side);
+                return lbm::launch_step_moments<decltype(P)::value>((int)((ts + k) & 1), a, c->hm.data(), side);
             });
             if (r) return r;
         }
@@ -1683,12 +1682,11 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
         }
         for (int64_t k = ns - 1; k >= 0 && rc == LBM_OK; --k) {
             const int64_t t = ts + k;
-            StepArgs a = make_args(c, t);
-            a.overlap = k < ns - 1 && overlaps(c);
             j.lam_next = (char *)lam + (size_t)((t + 1) & 1) * 27 * n * es;
             j.lam = (char *)lam + (size_t)(t & 1) * 27 * n * es;
             j.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
-            rc = dispatch(c, [&](auto P) { return lbm::launch_adjoint<decltype(P)::value>(a, j, c->stream); });
+            const bool overlap = k < ns - 1 && overlaps(c);
+            rc = dispatch(c, [&](auto P) { return lbm::launch_adjoint<decltype(P)::value>(overlap, j, c->stream); });
         }
         if (rc == LBM_OK) {
             const StepArgs a = make_args(c, ts);

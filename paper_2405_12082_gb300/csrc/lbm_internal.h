@@ -40,6 +40,7 @@ struct PairArgsBase {
     const StepTime *times;
     int64_t t;
     double *stats;
+    void *moments;           // EX_MOMENTS: [9][scells]
     int64_t dstride;
     int32_t tidx;
     float f16_scale, f16_inv;
@@ -68,7 +69,7 @@ constexpr int EVEN2_BLOCKS = 5;
 __host__ __device__ inline int odd_single_planes(int nz) { return nz < 3 ? nz : 2 + (nz & 1); }
 __host__ __device__ inline int odd_pair_groups(int nz, int zc) { return nz < 3 ? 0 : ((nz - 2) / 2 * 2 + zc - 1) / zc; }
 inline void fill_pair_args(PairArgsBase &o, const StepArgs &a) {
-    o.pops = a.pops; o.stride = a.stride; o.times = a.times; o.t = a.t; o.stats = a.stats; o.dstride = a.dstride;
+    o.pops = a.pops; o.stride = a.stride; o.times = a.times; o.t = a.t; o.stats = a.stats; o.moments = a.moments; o.dstride = a.dstride;
     o.tidx = a.tidx; o.zero = 0; o.f16_scale = a.f16_scale; o.f16_inv = a.f16_inv;
 }
 inline void fill_pair_member(PairMember &o, const Member &d) {
@@ -172,10 +173,9 @@ inline int default_variant_odd(int precision, int wall, int64_t stored_cells) {
 }
 // the shape the ablation collision models are compiled for (one plane per thread)
 inline int model_variant(int precision) { return precision == LBM_F64 ? 0 : 2; }
-// the shape of the adjoint's moment-storing recompute (256 x 4, one plane per thread:
-// two planes per thread measured 2 % slower there)
-constexpr int MOM_VARIANT = 0;
-inline int moments_variant(int) { return MOM_VARIANT; }
+// the shape of the adjoint's moment-storing steps: pairs of cells where the context has them
+// (shape 9), else 256 x 4 with one plane per thread (two planes measured 2 % slower there)
+constexpr int MOM_VARIANT = 0, MOM_VARIANT_PAIRS = 9;
 // whether the storage can run the shape at all (a staged shape also needs a compact pipe
 // layout whose row groups fit its segments: checked per context)
 inline bool step_variant_ok(int precision, int variant) {
@@ -207,14 +207,21 @@ cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, con
                         cudaStream_t s);
 
 // Forward step that also stores rho, u, s4..s8 into a.moments (adjoint recompute;
-// single half-way pipe, F32 or F64 storage, in the shape moments_variant).
+// single half-way pipe, F32 or F64 storage, in shape MOM_VARIANT or MOM_VARIANT_PAIRS).
 template <int P>
-cudaError_t launch_step_moments(int parity, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_step_moments(int parity, const StepArgs &a, const Member *hm, cudaStream_t s);
 
-// One backward step of the adjoint (see k_adjoint): 256-thread blocks, each thread
-// takes ADJ_ZC consecutive planes of one stored position (two planes measured 7 %
-// slower than one on GB300: the loop state spills at the kernel's register budget).
-constexpr int ADJ_ZC = 1;
+// One backward step of the adjoint (see k_adjoint): blocks of ADJ_THREADS threads, each taking
+// ADJ_ZC consecutive planes of one stored position in pairs (FP32) or one plane (FP64).
+constexpr int ADJ_THREADS = 128, ADJ_ZC = 2;
+struct AdjMember {
+    const int4 *cellinfo;
+    const void *gz_field;
+    int32_t nx, ny, nz, Ps;
+    uint32_t n;               // stored cells: the stride of the adjoint and moment fields
+    float gf[3], omegaf;
+    double g[3], omega;
+};
 struct AdjArgs {
     const void *lam_next;     // lambda_{t+1}, [27][cells] in the compute type
     void *lam;                // lambda_t (written)
@@ -222,15 +229,33 @@ struct AdjArgs {
     double *acc;              // [cells]: dJ/dg_z (accumulated, FP64, dense cells)
     void *acc_seg;            // [stored cells]: dJ/dg_z of the current segment (compute type;
                               // added into acc and cleared after each segment)
-    double *blockacc;         // [2][nblocks * 8]: objective and dJ/domega per warp (accumulated)
+    double *blockacc;         // [2][nblocks * warps]: objective and dJ/domega per warp (accumulated)
     int32_t objective;        // LBM_J_UBULK | LBM_J_WSS
     double kappa;             // UBULK: 1 / (T N_fluid)
     double wss;               // WSS: 2 / (T 2 pi R nz)
     float kappa_f, wss_f;     // the same in float
     int32_t nblocks;
+    uint32_t nb_plane, nb_mul, nb_shr;       // blocks per plane
+    uint32_t zero;            // 0 (see adjoint_cells)
+    uint32_t own[27], pull[27];              // element offsets, as in the odd step (see lbm_pair.cuh)
+    AdjMember one;
 };
+template <class S> __device__ __forceinline__ S adj_g(const AdjMember &d, int k) {
+    if constexpr (sizeof(S) == 4) return d.gf[k]; else return d.g[k];
+}
+template <class S> __device__ __forceinline__ S adj_omega(const AdjMember &d) {
+    if constexpr (sizeof(S) == 4) return d.omegaf; else return d.omega;
+}
+template <class S> __device__ __forceinline__ S adj_wss(const AdjArgs &j) {
+    if constexpr (sizeof(S) == 4) return j.wss_f; else return j.wss;
+}
+template <class S> __device__ __forceinline__ S adj_kappa(const AdjArgs &j) {
+    if constexpr (sizeof(S) == 4) return j.kappa_f; else return j.kappa;
+}
 template <int P>
-cudaError_t launch_adjoint(const StepArgs &a, const AdjArgs &j, cudaStream_t s);
+void prepare_adjoint(AdjArgs &j, const Member &d);
+template <int P>
+cudaError_t launch_adjoint(bool overlap, const AdjArgs &j, cudaStream_t s);
 // acc[dense cell] += acc_seg[stored cell]; acc_seg = 0 (member 0 of a, compact layout).
 template <int P>
 cudaError_t launch_flush_segment(const StepArgs &a, const Member &hm, const AdjArgs &j, cudaStream_t s);

@@ -18,9 +18,6 @@ namespace lbm {
 // the FP64 sums (sample steps); EX_MOMENTS stores rho, u and s4..s8 of the
 // pre-collision state for the adjoint sweep.  BS threads per block, register budget
 // for MINB resident blocks per SM.
-#ifndef LBM_ADJ_MIN_BLOCKS
-#define LBM_ADJ_MIN_BLOCKS 3
-#endif
 
 // Whether the step's populations travel in storage units (the scaled half format with the
 // default collision: the scale is applied inside collide, see there).
@@ -617,8 +614,9 @@ __global__ void k_force_tables(const Member *members, int m, R *ftab, R *ztab) {
 // ---- adjoint step ------------------------------------------------------------------------------
 // Reverse of step t of a single half-way pipe.  mu = S^T lambda_{t+1} gathers
 // lambda_i(x + c_i) when x + c_i is fluid and lambda_ibar(x) across a wall link (the
-// transpose of half-way bounce-back); the wall-shear objective adds 2 c_iz / (T A_w) on
-// wall links.  The collision is a function of rho, u and the raw shear moments m4..m8:
+// transpose of half-way bounce-back; in AA terms, direction ibar's odd-step read); the
+// wall-shear objective adds 2 c_iz / (T A_w) on wall links.  The collision is a function of
+// rho, u and the raw shear moments m4..m8:
 //   f*_j = w_j (rho P_j - 1) + (rho / 2) w_j g . grad_u P_j + (1 - omega) sum_k C_kj s_k,
 //   P_j = psi(c_jx, u_x) psi(c_jy, u_y) psi(c_jz, u_z) (normalised), s_k = m_k - rho e_k(u)
 //   + rho r_k(u, g) / 2,
@@ -627,182 +625,216 @@ __global__ void k_force_tables(const Member *members, int m, R *ftab, R *ztab) {
 // sum_j mu_j f*_j.  The sums over j of mu_j w_j times products of psi and its first two
 // u-derivatives are contracted axis by axis (z, then y, then x).  Per cell the FP64
 // accumulators collect the objective, dJ/dg_z(x) and dJ/domega.
-template <int P, int OBJ>
-__device__ __forceinline__ void adjoint_cell(const StepArgs &a, const AdjArgs &j, const Member &d, const CellPos &p,
-                                             typename Storage<P>::R &jterm, typename Storage<P>::R &wterm) {
-    using R = typename Storage<P>::R;
-    const uint32_t n = (uint32_t)d.scells, lc = (uint32_t)p.lc;
-    const R *M = static_cast<const R *>(j.moments) + lc;
-    const R rho = M[0], ux = M[n], uy = M[2 * n], uz = M[3 * n];
-    const R s4 = M[4 * n], s5 = M[5 * n], s6 = M[6 * n], s7 = M[7 * n], s8 = M[8 * n];
-    R gx, gy, gz;
-    acceleration<R>(d, p, a.t, st_of<R>(a, 0), gx, gy, gz);
-    const R om1 = R(1) - omega_of<R>(d);
-    const R half = R(0.5);
+//
+// One axis of a contraction, m the values at c = -1, 0, +1 (rest weight 4 times the others',
+// the common 1/6 left to the end): with P = m+ + m-, D = m+ - m-, E = 2 P - 4 m0, S = P + 4 m0
+//   sum psi m = S + 3 u (D + u E / 2),  sum psi' m = 3 (D + u E),  sum psi'' m = 3 E;
+// f1 and f2 return the last two without their factor 3.
+template <class R>
+struct AxisSum { R f0, f1, f2; };
+template <class R>
+__device__ __forceinline__ AxisSum<R> axis_sum(R mm, R m0, R mp, R u3, R uh, R u) {
+    const R P = add_(mp, mm), D = sub_(mp, mm);
+    const R E = fma_(lit<R>(-4), m0, add_(P, P)), S = fma_(lit<R>(4), m0, P);
+    return AxisSum<R>{fma_(u3, fma_(uh, E, D), S), fma_(u, E, D), E};
+}
+
+// One cell (R float or double, any plane) or the cells of planes z and z + 1 (R pf2, no
+// periodic wrap between them) of position r: jterm, wterm their objective and dJ/domega terms.
+// Bound by latency and issue (27 gathers, 9 moments, 27 stores per cell; the 50 MB fields live
+// in L2): pairs share the gather's addresses and halve the arithmetic's issue slots, and the
+// axis sums above take 162 operations where psi, psi', psi'' products took 220.  R = 24 pipe,
+// F32: 30 -> 22 us per step.
+template <int P, int OBJ, class R>
+__device__ __forceinline__ void adjoint_cells(const AdjArgs &j, const int4 ci, uint32_t r, int z, R &jterm, R &wterm) {
+    using S = typename scalar_of<R>::type;
+    constexpr bool TWO = std::is_same<R, pf2>::value;
+    const AdjMember &d = j.one;
+    const uint32_t ps = (uint32_t)d.Ps, nb = (uint32_t)ci.y, lc = r + (uint32_t)z * ps, n = d.n;
+    auto ld = [&](const S *q, uint32_t k) -> R {
+        if constexpr (TWO) return make_float2(q[k], q[k + ps]);
+        else return q[k];
+    };
+    auto st = [&](S *q, uint32_t k, R v) {
+        if constexpr (TWO) {
+            q[k] = v.x;
+            q[k + ps] = v.y;
+        } else {
+            q[k] = v;
+        }
+    };
+    const S *M = static_cast<const S *>(j.moments);
+    const R rho = ld(M, lc), ux = ld(M, n + lc), uy = ld(M, 2 * n + lc), uz = ld(M, 3 * n + lc);
+    const R s4 = ld(M, 4 * n + lc), s5 = ld(M, 5 * n + lc), s6 = ld(M, 6 * n + lc), s7 = ld(M, 7 * n + lc),
+            s8 = ld(M, 8 * n + lc);
+    const R gx = lit<R>(adj_g<S>(d, 0)), gy = lit<R>(adj_g<S>(d, 1));
+    R gz = lit<R>(adj_g<S>(d, 2));
+    if (d.gz_field != nullptr) {
+        const int64_t plane = (int64_t)d.nx * d.ny;
+        const S *q = static_cast<const S *>(d.gz_field) + (plane * z + (int64_t)(ci.x & 0xFFFF) * d.nx + ((uint32_t)ci.x >> 16));
+        if constexpr (TWO) gz = add_(gz, make_float2(q[0], q[plane]));
+        else gz = add_(gz, q[0]);
+    }
+    const R om1 = lit<R>(S(1) - adj_omega<S>(d));
+    const R half = lit<R>(S(0.5));
 
     // mu = S^T lambda_{t+1} (+ wall shear source)
-    const R wss = sizeof(R) == 4 ? (R)j.wss_f : (R)j.wss;
-    const R *ln = static_cast<const R *>(j.lam_next);
+    const S wss = adj_wss<S>(j);
+    const S *ln = static_cast<const S *>(j.lam_next);
     R mu[Q];
     sfor<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr int ib = opp_of(i);
-        const uint32_t push = i * n + (uint32_t)(p.lc + nb_offset<i>(p));
-        if constexpr (cx_of(i) == 0 && cy_of(i) == 0) {
-            mu[i] = ln[push];
+        constexpr int i = decltype(ic)::value, ib = opp_of(i), cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+        uint32_t pull = j.pull[ib];
+        if constexpr (!TWO && cz == -1) pull += z == 0 ? (uint32_t)d.nz * ps : 0u;
+        if constexpr (!TWO && cz == 1) pull -= z == d.nz - 1 ? (uint32_t)d.nz * ps : 0u;
+        if constexpr (cx == 0 && cy == 0) {
+            mu[i] = ld(ln, lc + (j.own[ib] + pull));
         } else {
-            const bool f = dst_is_fluid<i>(p);
-            mu[i] = ln[f ? push : ib * n + lc];
-            if constexpr (OBJ == LBM_J_WSS && cz_of(i) != 0)
-                if (!f) mu[i] += wss * R(cz_of(i));
+            const uint32_t f = (uint32_t)((int32_t)(nb << (31 - nbit(cx, cy))) >> 31);
+            const uint32_t dx = (cy == 0 ? 0u : (uint32_t)(cy < 0 ? ci.z : ci.w)) + (uint32_t)cx;
+            mu[i] = ld(ln, (lc + (f & dx)) + j.own[ib] + (f & pull));
+            if constexpr (OBJ == LBM_J_WSS && cz != 0)
+                if (!f) mu[i] = add_(mu[i], lit<R>(wss * S(cz)));
         }
     });
 
-    // axis factors psi, psi', psi'' at c = -1, 0, +1
-    R X0[3], X1[3], Y0[3], Y1[3], Z0[3], Z1[3];
-    auto fac = [&](R u, R (&F0)[3], R (&F1)[3]) {
-        const R u2 = u * u;
-        F0[1] = R(1) - R(1.5) * u2;
-        F0[0] = R(1) - R(3) * u + R(3) * u2;
-        F0[2] = R(1) + R(3) * u + R(3) * u2;
-        F1[1] = R(-3) * u;
-        F1[0] = R(-3) + R(6) * u;
-        F1[2] = R(3) + R(6) * u;
-    };
-    fac(ux, X0, X1);
-    fac(uy, Y0, Y1);
-    fac(uz, Z0, Z1);
-    const R D2[3] = {R(6), R(-3), R(6)};   // psi'' (same on every axis)
+    // q_k = sum_j mu_j C_kj (columns of (M^T)^{-1}), times 1 - omega
+    const R e12 = add_(mu[1], mu[2]), e34 = add_(mu[3], mu[4]), e56 = add_(mu[5], mu[6]);
+    const R q4 = mul_(lit<R>(S(0.25)), sub_(add_(mu[7], mu[10]), add_(mu[8], mu[9])));
+    const R q5 = mul_(lit<R>(S(0.25)), sub_(add_(mu[11], mu[14]), add_(mu[12], mu[13])));
+    const R q6 = mul_(lit<R>(S(0.25)), sub_(add_(mu[15], mu[18]), add_(mu[16], mu[17])));
+    const R q7 = mul_(lit<R>(S(1.0 / 6.0)), fma_(lit<R>(-2), e34, add_(e12, e56)));
+    const R q8 = mul_(lit<R>(S(1.0 / 6.0)), fma_(lit<R>(-2), e56, add_(e12, e34)));
+    wterm = neg_(fma_(q4, s4, fma_(q5, s5, fma_(q6, s6, fma_(q7, s7, mul_(q8, s8))))));
+    const R o4 = mul_(om1, q4), o5 = mul_(om1, q5), o6 = mul_(om1, q6), o7 = mul_(om1, q7), o8 = mul_(om1, q8);
 
-    // contraction over z: T0/T1/T2[a][b] = sum_c mu w Z0/Z1/Z2
-    R T0[3][3], T1[3][3], T2[3][3];
-#pragma unroll
-    for (int aa = 0; aa < 3; ++aa)
-#pragma unroll
-        for (int bb = 0; bb < 3; ++bb) T0[aa][bb] = T1[aa][bb] = T2[aa][bb] = R(0);
-    sfor<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr int aa = cx_of(i) + 1, bb = cy_of(i) + 1, cc = cz_of(i) + 1;
-        const R mw = mu[i] * R(w_of(i));
-        T0[aa][bb] += mw * Z0[cc];
-        T1[aa][bb] += mw * Z1[cc];
-        T2[aa][bb] += mw * D2[cc];
+    // contractions; Kabc: a, b, c derivatives along x, y, z
+    const R ux3 = mul_(lit<R>(3), ux), uy3 = mul_(lit<R>(3), uy), uz3 = mul_(lit<R>(3), uz);
+    const R uxh = mul_(half, ux), uyh = mul_(half, uy), uzh = mul_(half, uz);
+    AxisSum<R> Y0[3], Y1[3];          // per c_x: over z (derivative 0, 1), then y
+    R Y2[3];                          // second z derivative, plain in y
+    sfor<0, 3>([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        AxisSum<R> T[3];
+        sfor<0, 3>([&](auto bc) {
+            constexpr int b = decltype(bc)::value;
+            T[b] = axis_sum<R>(mu[dir_of(a - 1, b - 1, -1)], mu[dir_of(a - 1, b - 1, 0)], mu[dir_of(a - 1, b - 1, 1)], uz3, uzh, uz);
+        });
+        Y0[a] = axis_sum<R>(T[0].f0, T[1].f0, T[2].f0, uy3, uyh, uy);
+        Y1[a] = axis_sum<R>(T[0].f1, T[1].f1, T[2].f1, uy3, uyh, uy);
+        Y2[a] = axis_sum<R>(T[0].f2, T[1].f2, T[2].f2, uy3, uyh, uy).f0;
     });
-    // over y
-    R Y00[3], Y01[3], Y02[3], Y10[3], Y11[3], Y20[3];
-#pragma unroll
-    for (int aa = 0; aa < 3; ++aa) {
-        Y00[aa] = Y01[aa] = Y02[aa] = Y10[aa] = Y11[aa] = Y20[aa] = R(0);
-#pragma unroll
-        for (int bb = 0; bb < 3; ++bb) {
-            Y00[aa] += Y0[bb] * T0[aa][bb];
-            Y01[aa] += Y0[bb] * T1[aa][bb];
-            Y02[aa] += Y0[bb] * T2[aa][bb];
-            Y10[aa] += Y1[bb] * T0[aa][bb];
-            Y11[aa] += Y1[bb] * T1[aa][bb];
-            Y20[aa] += D2[bb] * T0[aa][bb];
-        }
-    }
-    // over x
-    R K000 = 0, K001 = 0, K002 = 0, K010 = 0, K011 = 0, K020 = 0, K100 = 0, K101 = 0, K110 = 0, K200 = 0;
-#pragma unroll
-    for (int aa = 0; aa < 3; ++aa) {
-        K000 += X0[aa] * Y00[aa];
-        K001 += X0[aa] * Y01[aa];
-        K002 += X0[aa] * Y02[aa];
-        K010 += X0[aa] * Y10[aa];
-        K011 += X0[aa] * Y11[aa];
-        K020 += X0[aa] * Y20[aa];
-        K100 += X1[aa] * Y00[aa];
-        K101 += X1[aa] * Y01[aa];
-        K110 += X1[aa] * Y10[aa];
-        K200 += D2[aa] * Y00[aa];
-    }
-    // q_k = sum_j mu_j C_kj (columns of (M^T)^{-1})
-    const R q4 = R(0.25) * (mu[7] + mu[10] - mu[8] - mu[9]);
-    const R q5 = R(0.25) * (mu[11] + mu[14] - mu[12] - mu[13]);
-    const R q6 = R(0.25) * (mu[15] + mu[18] - mu[16] - mu[17]);
-    const R q7 = (mu[1] + mu[2] + mu[5] + mu[6]) * R(1.0 / 6.0) - (mu[3] + mu[4]) * R(1.0 / 3.0);
-    const R q8 = (mu[1] + mu[2] + mu[3] + mu[4]) * R(1.0 / 6.0) - (mu[5] + mu[6]) * R(1.0 / 3.0);
+    const AxisSum<R> X00 = axis_sum<R>(Y0[0].f0, Y0[1].f0, Y0[2].f0, ux3, uxh, ux);
+    const AxisSum<R> X01 = axis_sum<R>(Y1[0].f0, Y1[1].f0, Y1[2].f0, ux3, uxh, ux);
+    const AxisSum<R> X10 = axis_sum<R>(Y0[0].f1, Y0[1].f1, Y0[2].f1, ux3, uxh, ux);
+    const R w0 = lit<R>(S(1.0 / 216.0)), w3 = lit<R>(S(1.0 / 72.0)), w9 = lit<R>(S(1.0 / 24.0));
+    const R K000 = mul_(w0, X00.f0), K100 = mul_(w3, X00.f1), K200 = mul_(w3, X00.f2);
+    const R K001 = mul_(w3, X01.f0), K101 = mul_(w9, X01.f1);
+    const R K010 = mul_(w3, X10.f0), K110 = mul_(w9, X10.f1);
+    const R K002 = mul_(w3, axis_sum<R>(Y2[0], Y2[1], Y2[2], ux3, uxh, ux).f0);
+    const R K011 = mul_(w9, axis_sum<R>(Y1[0].f1, Y1[1].f1, Y1[2].f1, ux3, uxh, ux).f0);
+    const R K020 = mul_(w3, axis_sum<R>(Y0[0].f2, Y0[1].f2, Y0[2].f2, ux3, uxh, ux).f0);
 
-    const R Arho = K000 + half * (gx * K100 + gy * K010 + gz * K001) +
-                   om1 * (q4 * (-ux * uy + half * (gy * ux + gx * uy)) + q5 * (-ux * uz + half * (gz * ux + gx * uz)) +
-                          q6 * (-uy * uz + half * (gz * uy + gy * uz)) + q7 * (-(ux * ux - uy * uy) + (gx * ux - gy * uy)) +
-                          q8 * (-(ux * ux - uz * uz) + (gx * ux - gz * uz)));
-    const R Aux = rho * (K100 + half * (gx * K200 + gy * K110 + gz * K101) +
-                         om1 * (q4 * (-uy + half * gy) + q5 * (-uz + half * gz) + (q7 + q8) * (R(-2) * ux + gx)));
-    const R Auy = rho * (K010 + half * (gx * K110 + gy * K020 + gz * K011) +
-                         om1 * (q4 * (-ux + half * gx) + q6 * (-uz + half * gz) + q7 * (R(2) * uy - gy)));
-    const R Auz = rho * (K001 + half * (gx * K101 + gy * K011 + gz * K002) +
-                         om1 * (q5 * (-ux + half * gx) + q6 * (-uy + half * gy) + q8 * (R(2) * uz - gz)));
-    const R irho = R(1) / rho;
-    const R kap = sizeof(R) == 4 ? (R)j.kappa_f : (R)j.kappa;
-    const R Bx = Aux * irho, By = Auy * irho;
-    const R Bz = Auz * irho + (OBJ == LBM_J_UBULK ? kap * irho : R(0));
-    const R vx = ux - half * gx, vy = uy - half * gy, vz = uz - half * gz;
-    const R base = Arho - (Bx * vx + By * vy + Bz * vz);
+    // v = u - g / 2 (the bare velocity); the shear part of A_rho is -(v_a v_b - g_a g_b / 4), of
+    // A_u minus 2 v or the other axis' v
+    const R hx = mul_(half, gx), hy = mul_(half, gy), hz = mul_(half, gz);
+    const R vx = sub_(ux, hx), vy = sub_(uy, hy), vz = sub_(uz, hz);
+    const R xx = fma_(vx, vx, neg_(mul_(hx, hx))), yy = fma_(vy, vy, neg_(mul_(hy, hy))), zz = fma_(vz, vz, neg_(mul_(hz, hz)));
+    R sh = mul_(o4, fma_(vx, vy, neg_(mul_(hx, hy))));
+    sh = fma_(o5, fma_(vx, vz, neg_(mul_(hx, hz))), sh);
+    sh = fma_(o6, fma_(vy, vz, neg_(mul_(hy, hz))), sh);
+    sh = fma_(o7, sub_(xx, yy), sh);
+    sh = fma_(o8, sub_(xx, zz), sh);
+    const R Arho = sub_(fma_(hx, K100, fma_(hy, K010, fma_(hz, K001, K000))), sh);
+    const R o78 = add_(o7, o8);
+    // A_u / rho
+    const R shx = fma_(o4, vy, fma_(o5, vz, mul_(mul_(lit<R>(2), o78), vx)));
+    const R shy = fma_(o4, vx, fma_(o6, vz, mul_(mul_(lit<R>(-2), o7), vy)));
+    const R shz = fma_(o5, vx, fma_(o6, vy, mul_(mul_(lit<R>(-2), o8), vz)));
+    const R Bx = sub_(fma_(hx, K200, fma_(hy, K110, fma_(hz, K101, K100))), shx);
+    const R By = sub_(fma_(hx, K110, fma_(hy, K020, fma_(hz, K011, K010))), shy);
+    const R Az = sub_(fma_(hx, K101, fma_(hy, K011, fma_(hz, K002, K001))), shz);
+    const R kap = lit<R>(adj_kappa<S>(j));
+    const R Bz = OBJ == LBM_J_UBULK ? fma_(kap, recip_(rho), Az) : Az;
+    const R base = sub_(Arho, fma_(Bx, vx, fma_(By, vy, mul_(Bz, vz))));
 
     // lambda_i = base + c_i . B + (1 - omega)(cx cy q4 + cx cz q5 + cy cz q6 + (cx^2 - cy^2) q7
     // + (cx^2 - cz^2) q8), split into one term per axis and the three cross terms; only the
     // terms with a non-zero lattice coefficient are added
-    const R o4 = om1 * q4, o5 = om1 * q5, o6 = om1 * q6, o7 = om1 * q7, o8 = om1 * q8;
-    const R axm = (o7 + o8) - Bx, axp = (o7 + o8) + Bx;     // cx = -1, +1
-    const R aym = -o7 - By, ayp = By - o7;
-    const R azm = -o8 - Bz, azp = Bz - o8;
-    R *lo = static_cast<R *>(j.lam);
-    sfor<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+    const R axm = sub_(o78, Bx), axp = add_(o78, Bx);     // cx = -1, +1
+    const R aym = neg_(add_(o7, By)), ayp = sub_(By, o7);
+    const R azm = neg_(add_(o8, Bz)), azp = sub_(Bz, o8);
+    S *lo = static_cast<S *>(j.lam);
+    // (the zero depends on the sums: no store address is formed before them)
+    uint32_t bits;
+    if constexpr (TWO) bits = __float_as_uint(K000.x);
+    else bits = (uint32_t)__float_as_int((float)K000);
+    const uint32_t wlc = lc + min(bits, j.zero);
+    sfor<0, 9>([&](auto kc) {
+        constexpr int k = decltype(kc)::value, cx = k % 3 - 1, cy = k / 3 - 1;
         R l = base;
-        if constexpr (cx == 1) l += axp;
-        if constexpr (cx == -1) l += axm;
-        if constexpr (cy == 1) l += ayp;
-        if constexpr (cy == -1) l += aym;
-        if constexpr (cz == 1) l += azp;
-        if constexpr (cz == -1) l += azm;
-        if constexpr (cx * cy == 1) l += o4;
-        if constexpr (cx * cy == -1) l -= o4;
-        if constexpr (cx * cz == 1) l += o5;
-        if constexpr (cx * cz == -1) l -= o5;
-        if constexpr (cy * cz == 1) l += o6;
-        if constexpr (cy * cz == -1) l -= o6;
-        lo[i * n + lc] = l;
+        if constexpr (cx == 1) l = add_(l, axp);
+        if constexpr (cx == -1) l = add_(l, axm);
+        if constexpr (cy == 1) l = add_(l, ayp);
+        if constexpr (cy == -1) l = add_(l, aym);
+        if constexpr (cx * cy == 1) l = add_(l, o4);
+        if constexpr (cx * cy == -1) l = sub_(l, o4);
+        R t5 = azp, t6 = azm;                             // cz = +1, -1
+        if constexpr (cx == 1) { t5 = add_(t5, o5); t6 = sub_(t6, o5); }
+        if constexpr (cx == -1) { t5 = sub_(t5, o5); t6 = add_(t6, o5); }
+        if constexpr (cy == 1) { t5 = add_(t5, o6); t6 = sub_(t6, o6); }
+        if constexpr (cy == -1) { t5 = sub_(t5, o6); t6 = add_(t6, o6); }
+        st(lo, j.own[dir_of(cx, cy, 0)] + wlc, l);
+        st(lo, j.own[dir_of(cx, cy, 1)] + wlc, add_(l, t5));
+        st(lo, j.own[dir_of(cx, cy, -1)] + wlc, add_(l, t6));
     });
 
     // accumulators: objective, dJ/dg_z, dJ/domega
-    jterm = R(0);
     if constexpr (OBJ == LBM_J_UBULK) {
-        jterm = kap * uz;
+        jterm = mul_(kap, uz);
     } else {
         // the wall is a cylinder, so (cx, cy, +1) and (cx, cy, -1) are wall links together:
         // their terms are summed as the difference f*(+1) - f*(-1), formed from the
         // closed-form differences psi(+1) - psi(-1) = 6 u_z and psi'(+1) - psi'(-1) = 6
         // (the rest weights cancel exactly instead of in floating point)
-        if (p.nb != 0x1FFu) {
-            const R dZ0 = R(6) * uz;
+        jterm = lit<R>(0);
+        if (nb != 0x1FFu) {
+            const R dZ0 = mul_(lit<R>(6), uz);
+            auto psi = [](auto cc, R u, R &f, R &f1) {
+                constexpr int c = decltype(cc)::value;
+                if constexpr (c == 0) {
+                    f = fma_(lit<R>(S(-1.5)), mul_(u, u), lit<R>(1));
+                    f1 = mul_(lit<R>(-3), u);
+                } else {
+                    f = fma_(lit<R>(3), fma_(u, u, c > 0 ? u : neg_(u)), lit<R>(1));
+                    f1 = fma_(lit<R>(6), u, lit<R>(3 * c));
+                }
+            };
             sfor<0, 9>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 constexpr int cx = k % 3 - 1, cy = k / 3 - 1;
                 if constexpr (cx != 0 || cy != 0) {
                     constexpr int ip = dir_of(cx, cy, 1);
-                    if (!dst_is_fluid<ip>(p)) {
-                        const R x0y0 = X0[cx + 1] * Y0[cy + 1];
-                        const R dP = x0y0 * dZ0;
-                        const R dG = (gx * X1[cx + 1] * Y0[cy + 1] + gy * X0[cx + 1] * Y1[cy + 1]) * dZ0 +
-                                     gz * x0y0 * R(6);
-                        R dshear = 0;
-                        if constexpr (cy == 0) dshear = R(cx) * R(0.5) * s5;
-                        if constexpr (cx == 0) dshear = R(cy) * R(0.5) * s6;
-                        jterm += wss * (R(w_of(ip)) * rho * (dP + half * dG) + om1 * dshear);
+                    if (!((nb >> nbit(cx, cy)) & 1u)) {
+                        R X0, X1, Yp, Yd;
+                        psi(std::integral_constant<int, cx>{}, ux, X0, X1);
+                        psi(std::integral_constant<int, cy>{}, uy, Yp, Yd);
+                        const R x0y0 = mul_(X0, Yp);
+                        const R dG = fma_(fma_(mul_(gx, X1), Yp, mul_(mul_(gy, X0), Yd)), dZ0, mul_(mul_(gz, x0y0), lit<R>(6)));
+                        R t = mul_(mul_(lit<R>(S(w_of(ip))), rho), fma_(half, dG, mul_(x0y0, dZ0)));
+                        if constexpr (cy == 0) t = fma_(om1, mul_(lit<R>(S(0.5 * cx)), s5), t);
+                        if constexpr (cx == 0) t = fma_(om1, mul_(lit<R>(S(0.5 * cy)), s6), t);
+                        jterm = fma_(lit<R>(wss), t, jterm);
                     }
                 }
             });
         }
     }
-    const R gterm = half * rho * K001 + om1 * half * rho * (q5 * ux + q6 * uy - R(2) * q8 * uz) + half * Auz +
-                    (OBJ == LBM_J_UBULK ? half * kap : R(0));
-    wterm = -(q4 * s4 + q5 * s5 + q6 * s6 + q7 * s7 + q8 * s8);
-    static_cast<R *>(j.acc_seg)[p.lc] += gterm;
+    const R hrho = mul_(half, rho);
+    R gterm = fma_(hrho, add_(K001, Az), mul_(hrho, fma_(o5, ux, fma_(o6, uy, mul_(mul_(lit<R>(-2), o8), uz)))));
+    if constexpr (OBJ == LBM_J_UBULK) gterm = fma_(half, kap, gterm);
+    S *seg = static_cast<S *>(j.acc_seg);
+    st(seg, lc, add_(ld(seg, lc), gterm));
 }
 
 // End of a segment of the reverse sweep: its dJ/dg_z sums join the FP64 totals (dense cells).
@@ -819,35 +851,36 @@ __global__ void k_flush_segment(const Member *members, R *acc_seg, double *acc) 
     acc_seg[s] = R(0);
 }
 
-// One thread per ADJ_ZC consecutive planes of one stored position; the objective and
-// dJ/domega terms are summed per warp in a fixed order and added to the warp's own FP64
-// slots (deterministic), dJ/dg_z per cell.
+// FP32: planes 1 .. nz - 2 in pairs, ADJ_ZC / 2 pairs per thread, after the planes taken singly (as
+// in k_odd2); FP64: every plane singly.  The objective and dJ/domega terms are summed per warp
+// in a fixed order and added to the warp's own FP64 slots (deterministic), dJ/dg_z per cell.
 template <int P, int OBJ>
-__global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint(const __grid_constant__ StepArgs a,
-                                                                     const AdjArgs j) {
-    using R = typename Storage<P>::R;
+__global__ void __launch_bounds__(ADJ_THREADS, P == LBM_F64 ? 3 : 4) k_adjoint(const __grid_constant__ AdjArgs j) {
+    using S = typename Storage<P>::R;
     release_next_step();
-    const Member &d = a.members[0];
-    const uint32_t local = blockIdx.x * 256u + threadIdx.x;
-    const uint32_t nzg = (uint32_t)(d.nz + ADJ_ZC - 1) / ADJ_ZC;
-    R x0 = 0, x1 = 0;
-    if (local < (uint32_t)d.Ps * nzg) {
-        const uint32_t zg = fastdiv(local, d.ps_mul, d.ps_shr);
-        const uint32_t r = local - zg * (uint32_t)d.Ps;
-        CellPos p;
-        const bool fluid = cell_from_storage(d, zg * ADJ_ZC * (uint32_t)d.Ps + r, p);
-        await_previous_step();
-        if (fluid) {
+    const AdjMember &d = j.one;
+    const uint32_t zg = fastdiv(blockIdx.x, j.nb_mul, j.nb_shr);
+    const uint32_t r = (blockIdx.x - zg * j.nb_plane) * ADJ_THREADS + threadIdx.x;
+    const int4 ci = r < (uint32_t)d.Ps ? d.cellinfo[r] : make_int4(-1, 0, 0, 0);
+    await_previous_step();
+    S x0 = 0, x1 = 0;
+    if (ci.x != -1) {
+        const int singles = P == LBM_F64 ? d.nz : odd_single_planes(d.nz);
+        if ((int)zg < singles) {
+            const int z = P == LBM_F64 ? (int)zg : (zg == 0 ? 0 : d.nz - (int)zg);
+            adjoint_cells<P, OBJ, S>(j, ci, r, z, x0, x1);
+        } else if constexpr (P != LBM_F64) {
 #pragma unroll 1
-            for (int k = 0; k < ADJ_ZC; ++k) {
-                if (k > 0) {
-                    if (p.z + 1 >= d.nz) break;
-                    next_plane(d, p);
-                }
-                R y0, y1;
-                adjoint_cell<P, OBJ>(a, j, d, p, y0, y1);
-                x0 += y0;
-                x1 += y1;
+            for (int k = 0; k < ADJ_ZC / 2; ++k) {
+                const int z = 1 + ((int)zg - singles) * ADJ_ZC + 2 * k;
+                if (z + 2 >= d.nz) break;
+                uint32_t rr = r;
+                int4 cj = ci;
+                asm volatile("" : "+r"(rr), "+r"(cj.x), "+r"(cj.y), "+r"(cj.z), "+r"(cj.w));    // nothing of a pass outlives it
+                pf2 y0, y1;
+                adjoint_cells<P, OBJ, pf2>(j, cj, rr, z, y0, y1);
+                x0 += y0.x + y0.y;
+                x1 += y1.x + y1.y;
             }
         }
     }
@@ -859,10 +892,9 @@ __global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint(const __gri
         x1 += __shfl_down_sync(0xFFFFFFFFu, x1, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        await_previous_step();               // (a warp past the last position)
-        const int64_t wslot = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+        const int64_t wslot = (int64_t)blockIdx.x * (ADJ_THREADS / 32) + (threadIdx.x >> 5);
         j.blockacc[wslot] += (double)x0;
-        j.blockacc[(int64_t)j.nblocks * 8 + wslot] += (double)x1;
+        j.blockacc[(int64_t)j.nblocks * (ADJ_THREADS / 32) + wslot] += (double)x1;
     }
 }
 
@@ -995,16 +1027,21 @@ void fill_pull(PairArgsOne &o, uint32_t stride, uint32_t ps, std::integer_sequen
     }
 }
 
+template <int V>
+void fill_pair_one(PairArgsOne &o, const StepArgs &a, const Member *hm) {
+    fill_pair_args(o, a);
+    fill_pair_member(o.one, hm[0]);
+    o.stf[0] = a.stf[0];
+    o.nb_plane = (uint32_t)((hm[0].Ps + STEP_SHAPES[V].pt - 1) / STEP_SHAPES[V].pt);
+    fastdiv_setup(o.nb_plane, o.nb_mul, o.nb_shr);
+    fill_pull(o, (uint32_t)a.stride, (uint32_t)hm[0].Ps, std::make_integer_sequence<int, Q>{});
+}
+
 template <int P, int V>
 cudaError_t launch_pair(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, cudaStream_t s) {
     if (a.n_members == 1) {
         PairArgsOne o;
-        fill_pair_args(o, a);
-        fill_pair_member(o.one, hm[0]);
-        o.stf[0] = a.stf[0];
-        o.nb_plane = (uint32_t)((hm[0].Ps + STEP_SHAPES[V].pt - 1) / STEP_SHAPES[V].pt);
-        fastdiv_setup(o.nb_plane, o.nb_mul, o.nb_shr);
-        fill_pull(o, (uint32_t)a.stride, (uint32_t)hm[0].Ps, std::make_integer_sequence<int, Q>{});
+        fill_pair_one<V>(o, a, hm);
         return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, a.overlap, o, s)
                                    : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, a.overlap, o, s);
     }
@@ -1076,10 +1113,20 @@ cudaError_t launch_step(int wall, int parity, bool stats, const StepArgs &a, con
 
 // Forward step of a single half-way pipe that also stores the adjoint moments (F32, F64).
 template <int P>
-cudaError_t launch_step_moments(int parity, const StepArgs &a, cudaStream_t s) {
+cudaError_t launch_step_moments(int parity, const StepArgs &a, const Member *hm, cudaStream_t s) {
+    if constexpr (P == LBM_F32) {
+        if (a.pairs) {
+            PairArgsOne o;
+            constexpr StepShape S = STEP_SHAPES[MOM_VARIANT_PAIRS];
+            fill_pair_one<MOM_VARIANT_PAIRS>(o, a, hm);
+            if (parity == 0)
+                return launch_step_kernel<PairArgsOne>(k_even2<P, LBM_HALFWAY, EX_MOMENTS, 128, EVEN2_BLOCKS, PairArgsOne>, a.nblocks_total, 128, a.overlap, o, s);
+            return launch_step_kernel<PairArgsOne>(k_odd2<P, LBM_HALFWAY, EX_MOMENTS, S.pt, S.pb, S.pz, PairArgsOne>, a.nblocks_total, S.pt, a.overlap, o, s);
+        }
+    }
     if constexpr (P == LBM_F64 || P == LBM_F32) {
         constexpr int BS = P == LBM_F64 ? STEP_SHAPE_F64.threads : 256, MINB = P == LBM_F64 ? STEP_SHAPE_F64.min_blocks : 4;
-        constexpr int ZC = (P == LBM_F64) ? 1 : STEP_SHAPES[MOM_VARIANT].zc;
+        constexpr int ZC = 1;
         if (parity == 0)
             return launch_step_kernel<StepArgs>(k_step<P, 0, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
         return launch_step_kernel<StepArgs>(k_step<P, 1, LBM_HALFWAY, EX_MOMENTS, BS, MINB, MODEL_MRT_H6, ZC>, a.nblocks_total, BS, a.overlap, a, s);
@@ -1102,15 +1149,42 @@ cudaError_t launch_sum_columns(const double *base, int64_t n, int nv, double *pa
 }
 
 template <int P>
-cudaError_t launch_adjoint(const StepArgs &a, const AdjArgs &j, cudaStream_t s) {
+cudaError_t launch_adjoint(bool overlap, const AdjArgs &j, cudaStream_t s) {
     if constexpr (P == LBM_F64 || P == LBM_F32) {
-        cudaLaunchAttribute at[1];
-        cudaLaunchConfig_t cfg = step_config(j.nblocks, 256, a.overlap, at, s);
-        if (j.objective == LBM_J_UBULK) return cudaLaunchKernelEx(&cfg, k_adjoint<P, LBM_J_UBULK>, a, j);
-        return cudaLaunchKernelEx(&cfg, k_adjoint<P, LBM_J_WSS>, a, j);
+        if (j.objective == LBM_J_UBULK) return launch_step_kernel<AdjArgs>(k_adjoint<P, LBM_J_UBULK>, j.nblocks, ADJ_THREADS, overlap, j, s);
+        return launch_step_kernel<AdjArgs>(k_adjoint<P, LBM_J_WSS>, j.nblocks, ADJ_THREADS, overlap, j, s);
     } else {
         return cudaErrorNotSupported;
     }
+}
+
+// Everything about the pipe and the launch that stays the same over the sweep.
+template <int... I>
+void fill_adjoint_index(AdjArgs &j, std::integer_sequence<int, I...>) {
+    constexpr int jump[] = {(opp_of(I) - I)...}, cz[] = {cz_of(I)...};
+    for (int i = 0; i < Q; ++i) {
+        j.own[i] = (uint32_t)i * j.one.n;
+        j.pull[i] = (uint32_t)jump[i] * j.one.n - (uint32_t)cz[i] * (uint32_t)j.one.Ps;
+    }
+}
+template <int P>
+void prepare_adjoint(AdjArgs &j, const Member &d) {
+    AdjMember &o = j.one;
+    o.cellinfo = d.cellinfo;
+    o.gz_field = d.gz_field;
+    o.nx = d.nx; o.ny = d.ny; o.nz = d.nz; o.Ps = d.Ps;
+    o.n = (uint32_t)d.scells;
+    for (int k = 0; k < 3; ++k) {
+        o.g[k] = d.g[k];
+        o.gf[k] = d.gf[k];
+    }
+    o.omega = d.omega;
+    o.omegaf = d.omegaf;
+    j.zero = 0;
+    j.nb_plane = (uint32_t)((d.Ps + ADJ_THREADS - 1) / ADJ_THREADS);
+    fastdiv_setup(j.nb_plane, j.nb_mul, j.nb_shr);
+    j.nblocks = (int32_t)(j.nb_plane * (P == LBM_F64 ? d.nz : odd_single_planes(d.nz) + odd_pair_groups(d.nz, ADJ_ZC)));
+    fill_adjoint_index(j, std::make_integer_sequence<int, Q>{});
 }
 
 template <int P>
@@ -1207,8 +1281,9 @@ cudaError_t launch_modes(int wall, int parity, const StepArgs &a, const Member &
     namespace lbm {                                                                                     \
     template cudaError_t launch_step<P>(int, int, bool, const StepArgs &, const Member *, int,            \
                                          cudaStream_t);                                                  \
-    template cudaError_t launch_step_moments<P>(int, const StepArgs &, cudaStream_t);                    \
-    template cudaError_t launch_adjoint<P>(const StepArgs &, const AdjArgs &, cudaStream_t);             \
+    template cudaError_t launch_step_moments<P>(int, const StepArgs &, const Member *, cudaStream_t);     \
+    template cudaError_t launch_adjoint<P>(bool, const AdjArgs &, cudaStream_t);                         \
+    template void prepare_adjoint<P>(AdjArgs &, const Member &);                                         \
     template cudaError_t launch_flush_segment<P>(const StepArgs &, const Member &, const AdjArgs &,       \
                                                  cudaStream_t);                                          \
     template cudaError_t launch_sum_columns<P>(const double *, int64_t, int, double *, int, double *,    \

@@ -177,7 +177,19 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
             sfor<0, Q>([&](auto jc) { store(jc, v[decltype(jc)::value]); });
         }
     } else {
-        mm = collide_mrt<pf2, SC, true, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr, store, act);
+        pf2 sk[5];
+        mm = collide_mrt<pf2, SC, true, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
+                                                      EXTRA == EX_MOMENTS ? sk : nullptr, store, act);
+        if constexpr (EXTRA == EX_MOMENTS) {
+            pf2 *mo = reinterpret_cast<pf2 *>(static_cast<float *>(a.moments) + lc);
+            const int64_t n = d.scells >> 1;
+            mo[0] = mm.rho;
+            mo[n] = mm.ux;
+            mo[2 * n] = mm.uy;
+            mo[3 * n] = mm.uz;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) mo[(4 + k) * n] = sk[k];
+        }
     }
     if constexpr (EXTRA == EX_STATS) {
         const int64_t cell = d.doff + plane * z + col;
@@ -296,7 +308,23 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
             store(jc, f);
         });
     } else {
-        mm = collide_mrt<R, SC, false, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr, store);
+        R sk[5];
+        mm = collide_mrt<R, SC, false, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
+                                                     EXTRA == EX_MOMENTS ? sk : nullptr, store);
+        if constexpr (EXTRA == EX_MOMENTS) {
+            float *mo = static_cast<float *>(a.moments) + (own - (uint32_t)d.off);
+            const R out[9] = {mm.rho, mm.ux, mm.uy, mm.uz, sk[0], sk[1], sk[2], sk[3], sk[4]};
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                float *q = mo + k * d.scells;
+                if constexpr (TWO) {
+                    q[0] = out[k].x;
+                    q[d.Ps] = out[k].y;
+                } else {
+                    q[0] = out[k];
+                }
+            }
+        }
     }
     if constexpr (EXTRA == EX_STATS) {
         double *s = a.stats + d.doff + plane * z + col;
