@@ -55,10 +55,12 @@ struct PairArgsOne : PairArgsBase {
 };
 struct PairArgsMany : PairArgsBase {
     static constexpr bool kOne = false;
-    const Member *members;
     int32_t n_members;
     float stf[LBM_MAX_MEMBERS];
     int32_t block0[LBM_MAX_MEMBERS + 1];
+    uint32_t nb_plane[LBM_MAX_MEMBERS], nb_mul[LBM_MAX_MEMBERS], nb_shr[LBM_MAX_MEMBERS];
+    uint32_t own[27], pull[27];              // pull without the plane offset
+    PairMember many[LBM_MAX_MEMBERS];
 };
 // Resident blocks of 128 threads the even pair kernel's registers are cut for (5: 96 registers).
 // R = 96 / R = 48 pipe, fraction of the copy bandwidth: F32 5 blocks 0.992 / 0.907 (4: 0.987 /

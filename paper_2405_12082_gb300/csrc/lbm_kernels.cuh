@@ -1018,8 +1018,8 @@ cudaError_t launch_pair_args(int parity, bool stats, int blocks, bool overlap, c
 }
 
 // (the lattice functions folded by the compiler: evaluated per launch they took 4 us)
-template <int... I>
-void fill_pull(PairArgsOne &o, uint32_t stride, uint32_t ps, std::integer_sequence<int, I...>) {
+template <class A, int... I>
+void fill_pull(A &o, uint32_t stride, uint32_t ps, std::integer_sequence<int, I...>) {
     constexpr int jump[] = {(opp_of(I) - I)...}, cz[] = {cz_of(I)...};
     for (int i = 0; i < Q; ++i) {
         o.own[i] = (uint32_t)i * stride;
@@ -1047,9 +1047,14 @@ cudaError_t launch_pair(int wall, int parity, bool stats, const StepArgs &a, con
     }
     PairArgsMany o;
     fill_pair_args(o, a);
-    o.members = a.members;
     o.n_members = a.n_members;
-    for (int m = 0; m < a.n_members; ++m) o.stf[m] = a.stf[m];
+    fill_pull(o, (uint32_t)a.stride, 0u, std::make_integer_sequence<int, Q>{});
+    for (int m = 0; m < a.n_members; ++m) {
+        o.stf[m] = a.stf[m];
+        fill_pair_member(o.many[m], hm[m]);
+        o.nb_plane[m] = (uint32_t)((hm[m].Ps + STEP_SHAPES[V].pt - 1) / STEP_SHAPES[V].pt);
+        fastdiv_setup(o.nb_plane[m], o.nb_mul[m], o.nb_shr[m]);
+    }
     for (int m = 0; m <= a.n_members; ++m) o.block0[m] = a.block0[m];
     return wall == LBM_BOUZIDI ? launch_pair_args<P, V, LBM_BOUZIDI>(parity, stats, a.nblocks_total, a.overlap, o, s)
                                : launch_pair_args<P, V, LBM_HALFWAY>(parity, stats, a.nblocks_total, a.overlap, o, s);

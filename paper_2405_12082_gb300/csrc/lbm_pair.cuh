@@ -52,8 +52,8 @@ template <> struct PairStorage<LBM_BF16> {
 };
 
 // ---- what a block works on --------------------------------------------------------------
-// A context with one pipe passes its member in the kernel parameters (every base address is
-// then uniform); an ensemble looks it up by block.
+// Members travel in the kernel parameters (their fields are then constants of the launch, not
+// loads); an ensemble looks its member up by block.
 struct PairTask {
     uint32_t local;      // block index inside the member
     int m;
@@ -74,7 +74,7 @@ __device__ __forceinline__ PairTask pair_task(const A &a) {
 template <class A>
 __device__ __forceinline__ const auto &pair_member(const A &a, int m) {
     if constexpr (A::kOne) return a.one;
-    else return a.members[m];
+    else return a.many[m];
 }
 template <class A>
 __device__ __forceinline__ float pair_st(const A &a, int m) {
@@ -205,13 +205,12 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
 // and the difference are constants of the context (kOne: kernel parameters).
 template <int I, class A, class D>
 __device__ __forceinline__ uint32_t own_at(const A &a, const D &d) {
-    if constexpr (A::kOne) return a.own[I];
-    else return (uint32_t)I * (uint32_t)a.stride;
+    return a.own[I];
 }
 template <int I, class A, class D>
 __device__ __forceinline__ uint32_t pull_at(const A &a, const D &d) {       // less the own part
     if constexpr (A::kOne) return a.pull[I];
-    else return (uint32_t)(opp_of(I) - I) * (uint32_t)a.stride - (uint32_t)(cz_of(I) * d.Ps);
+    else return a.pull[I] - (uint32_t)(cz_of(I) * d.Ps);       // (the members' planes differ)
 }
 
 // One cell (R float, at any plane) or the cells of planes z and z + 1 (R pf2, 1 <= z, z + 2 <
@@ -349,8 +348,8 @@ __global__ void __launch_bounds__(BS, MINB) k_odd2(const __grid_constant__ A a) 
         nb_plane = a.nb_plane;
         zg = fastdiv(tk.local, a.nb_mul, a.nb_shr);
     } else {
-        nb_plane = ((uint32_t)d.Ps + BS - 1) / BS;
-        zg = tk.local / nb_plane;
+        nb_plane = a.nb_plane[tk.m];
+        zg = fastdiv(tk.local, a.nb_mul[tk.m], a.nb_shr[tk.m]);
     }
     const uint32_t r = (tk.local - zg * nb_plane) * BS + threadIdx.x;
     if (r >= (uint32_t)d.Ps) return;
