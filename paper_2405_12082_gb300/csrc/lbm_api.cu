@@ -571,7 +571,7 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         if (sk >= 0) {
             blk += (int64_t)d.nsg[sk] * d.nz;        // staged: one tile per (plane, row group)
         } else if (pairs && (t & 1) == 0) {
-            blk += ceil_div(d.scells / 2, 128);      // pairs of stored positions
+            blk += ceil_div(d.scells / (2 * lbm::even_pairs(c->precision, c->wall)), 128);
         } else if (pairs) {
             blk += ceil_div(d.Ps, lbm::STEP_SHAPES[v].pt) *
                    (lbm::odd_single_planes(d.nz) + lbm::odd_pair_groups(d.nz, lbm::STEP_SHAPES[v].pz));

@@ -64,8 +64,10 @@ struct PairArgsMany : PairArgsBase {
 };
 // Resident blocks of 128 threads the even pair kernel's registers are cut for (5: 96 registers).
 // R = 96 / R = 48 pipe, fraction of the copy bandwidth: F32 5 blocks 0.992 / 0.907 (4: 0.987 /
-// 0.897, 6: 0.963 / 0.876), F16S 0.773 / 0.659 (4: 0.70 / 0.61), BF16 0.715 / 0.607.
-constexpr int EVEN2_BLOCKS = 5;
+// 0.897, 6: 0.963 / 0.876).
+// The 16-bit formats' two pairs per thread take 128 registers (4 blocks).
+constexpr int even_pairs(int precision, int wall) { return precision == LBM_F32 || wall == LBM_BOUZIDI ? 1 : 2; }
+template <int P, int WALL> constexpr int EVEN2_BLOCKS = even_pairs(P, WALL) == 1 ? 5 : 4;
 // Planes the odd pair kernel takes singly (0, nz - 1 and, for odd nz > 2, nz - 2), and its plane
 // groups of zc planes (the pairs 1 .. nz - 2) after them.
 __host__ __device__ inline int odd_single_planes(int nz) { return nz < 3 ? nz : 2 + (nz & 1); }

@@ -84,31 +84,18 @@ template <class A>
 __device__ __forceinline__ int64_t pair_t(const A &a) { return a.times ? a.times[a.tidx].t : a.t; }
 
 // ---- even step ----------------------------------------------------------------------------
-template <int P, int WALL, int EXTRA, int BS, int MINB, class A>
-__global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a) {
+// The pair at stored positions lc, lc + 1 (plane z, position r, table entry pi with its first
+// cell fluid), whose populations are in raw.
+template <int P, int WALL, int EXTRA, class A, class D>
+__device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_t lc, uint32_t z, uint32_t r, uint32_t pi,
+                                          const typename PairStorage<P>::V (&raw)[Q]) {
     using PS = PairStorage<P>;
     using T = typename PS::T;
     using V = typename PS::V;
     constexpr bool SC = P == LBM_F16S;
-    release_next_step();
-    const PairTask tk = pair_task(a);
-    const auto &d = pair_member(a, tk.m);
-    const uint32_t pair = tk.local * BS + threadIdx.x;
-    if (pair >= (uint32_t)(d.scells >> 1)) return;
-    const uint32_t lc = 2 * pair;
     char *const base = static_cast<char *>(a.pops);
     const uint64_t stb = (uint64_t)a.stride * sizeof(T);
     const uint32_t vo = ((uint32_t)d.off + lc) * (uint32_t)sizeof(T);
-    const uint32_t z = fastdiv(lc, d.ps_mul, d.ps_shr);
-    const uint32_t r = lc - z * (uint32_t)d.Ps;
-    const uint32_t pi = d.pairinfo[r >> 1];
-    await_previous_step();
-    V raw[Q];
-    sfor<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        raw[i] = *reinterpret_cast<const V *>(base + i * stb + vo);
-    });
-    if (!(pi & PAIR_A)) return;                 // both positions are padding
     const uint32_t col = pi >> PAIR_SHIFT;
     const pf2 act = make_float2(1.f, (pi & PAIR_B) ? 1.f : 0.f);
     // acceleration (see acceleration())
@@ -120,7 +107,7 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
         if (pi & PAIR_B) gz.y += q[1];
     }
     if (d.trig && pair_t(a) < d.t_end) {
-        const float st = pair_st(a, tk.m);
+        const float st = pair_st(a, m);
         const float *zt = static_cast<const float *>(d.ztab);
         const float2 *ft = reinterpret_cast<const float2 *>(d.ftabc) + (r >> 1);
         const pf2 sc = lit<pf2>(st * zt[z]), ss = lit<pf2>(st * zt[d.nz + z]);
@@ -195,6 +182,54 @@ __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a)
         const int64_t cell = d.doff + plane * z + col;
         add_stats(a.stats + cell, a.dstride, (double)mm.uz.x);
         if (pi & PAIR_B) add_stats(a.stats + cell + 1, a.dstride, (double)mm.uz.y);
+    }
+}
+
+// Two pairs per thread in the 16-bit formats with half-way walls (even_pairs): one 8-byte access
+// loads a population of four cells, so the second pair's values wait in 27 registers while the
+// first is collided, and the addresses serve both (R = 96 pipe: BF16 750 -> 662 us, F16S 687 ->
+// 681).  In F32 the second pair would take 54 registers, and with Bouzidi walls the outputs of a
+// pair are held as well (860 -> 1,002 us in F16S): one pair there.
+template <int P, int WALL, int EXTRA, int BS, int MINB, class A>
+__global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a) {
+    using PS = PairStorage<P>;
+    using T = typename PS::T;
+    using V = typename PS::V;
+    constexpr int NP = even_pairs(P, WALL);
+    release_next_step();
+    const PairTask tk = pair_task(a);
+    const auto &d = pair_member(a, tk.m);
+    const uint32_t group = tk.local * BS + threadIdx.x;
+    if (group >= (uint32_t)(d.scells / (2 * NP))) return;
+    const uint32_t lc = 2 * NP * group;
+    const char *const base = static_cast<const char *>(a.pops);
+    const uint64_t stb = (uint64_t)a.stride * sizeof(T);
+    const uint32_t vo = ((uint32_t)d.off + lc) * (uint32_t)sizeof(T);
+    const uint32_t z = fastdiv(lc, d.ps_mul, d.ps_shr);
+    const uint32_t r = lc - z * (uint32_t)d.Ps;
+    if constexpr (NP == 1) {
+        const uint32_t pi = d.pairinfo[r >> 1];
+        await_previous_step();
+        V raw[Q];
+        sfor<0, Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            raw[i] = *reinterpret_cast<const V *>(base + i * stb + vo);
+        });
+        if (pi & PAIR_A) even_pair<P, WALL, EXTRA>(a, d, tk.m, lc, z, r, pi, raw);
+    } else {
+        const uint2 pi = *reinterpret_cast<const uint2 *>(d.pairinfo + (r >> 1));
+        await_previous_step();
+        V first[Q], second[Q];
+        sfor<0, Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            const uint2 w = *reinterpret_cast<const uint2 *>(base + i * stb + vo);
+            first[i] = *reinterpret_cast<const V *>(&w.x);
+            second[i] = *reinterpret_cast<const V *>(&w.y);
+        });
+        // (a row's cells come before its padding: without a cell in the first pair the second has none)
+        if (!(pi.x & PAIR_A)) return;
+        even_pair<P, WALL, EXTRA>(a, d, tk.m, lc, z, r, pi.x, first);
+        if (pi.y & PAIR_A) even_pair<P, WALL, EXTRA>(a, d, tk.m, lc + 2, z, r + 2, pi.y, second);
     }
 }
 
