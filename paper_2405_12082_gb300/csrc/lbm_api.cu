@@ -516,11 +516,6 @@ int variant_at(const lbm_ctx *c, int64_t t) { return (t & 1) ? c->variant_odd : 
 // against 3.0, 110 k cells 5.6 against 4.8 (F32, steps in a row on the GPU).
 constexpr int64_t PAIRS_MIN_CELLS = 60000;
 
-// Whether a step may start while the one before it drains.  Not in FP64: those steps are bound
-// by the FP64 units of each SM, and blocks that arrive early pack onto the SMs the running step
-// leaves free (20 x 20 x 64 pipe: 21 us per step apart, 38 us overlapped).
-bool overlaps(const lbm_ctx *c) { return c->precision != LBM_F64; }
-
 // Whether the steps of the shapes of several planes per thread run on pairs of cells
 // (lbm_pair.cuh): F32 or 16-bit storage, the default model, every member compact and its
 // columns within the pair table's index range.
@@ -1039,7 +1034,7 @@ namespace {
 int step_direct(lbm_ctx *c, bool overlap = false) {
     const bool stats = c->stats && c->stats_every > 0 && (c->t % c->stats_every == 0);
     StepArgs a = make_args(c, c->t);
-    a.overlap = overlap && !c->prof && overlaps(c);
+    a.overlap = overlap && !c->prof;
     if (c->skip_tile >= 0 && lbm::staged_of(variant_at(c, c->t)) >= 0) {
         a.skip_tile = c->skip_tile;
         c->skip_tile = -1;
@@ -1094,7 +1089,7 @@ int build_graph(lbm_ctx *c) {
         StepArgs &a = ap[k & 1];
         a.times = c->d_times;
         a.tidx = k;
-        a.overlap = k > 0 && overlaps(c);
+        a.overlap = k > 0;
         const bool stats = every > 0 && (k % every == 0);
         const int v = variant_at(c, k);
         switch (c->precision) {
@@ -1612,7 +1607,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
             c->variant = c->variant_odd = c->stride >= PAIRS_MIN_CELLS && pairs_of(c) ? lbm::MOM_VARIANT_PAIRS : lbm::MOM_VARIANT;
             for (int64_t k = 0; k < ns && rc == LBM_OK; ++k) {
                 StepArgs a = make_args(c, c->t);
-                a.overlap = k > 0 && overlaps(c);
+                a.overlap = k > 0;
                 a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
                 rc = dispatch(c, [&](auto P) {
                     return lbm::launch_step_moments<decltype(P)::value>((int)(c->t & 1), a, c->hm.data(), c->stream);
@@ -1662,7 +1657,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
         if (ce != cudaSuccess) return cuda_err(c, ce, "checkpoint restore");
         for (int64_t k = 0; k < ns; ++k) {
             StepArgs a = make_args(c, ts + k);
-            a.overlap = k > 0 && overlaps(c);
+            a.overlap = k > 0;
             a.pops = work;
             a.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
             const int r = dispatch(c, [&](auto P) {
@@ -1685,7 +1680,7 @@ int lbm_adjoint(lbm_ctx *c, int64_t T, int32_t objective, int64_t checkpoint_eve
             j.lam_next = (char *)lam + (size_t)((t + 1) & 1) * 27 * n * es;
             j.lam = (char *)lam + (size_t)(t & 1) * 27 * n * es;
             j.moments = (char *)mom + (size_t)(sgm & 1) * mom_seg + (size_t)k * 9 * n * es;
-            const bool overlap = k < ns - 1 && overlaps(c);
+            const bool overlap = k < ns - 1;
             rc = dispatch(c, [&](auto P) { return lbm::launch_adjoint<decltype(P)::value>(overlap, j, c->stream); });
         }
         if (rc == LBM_OK) {
