@@ -517,7 +517,7 @@ def run_ours(args):
                      "frac": achieved / peak if achieved else None,
                      "traffic": profiled_traffic(args.precision, args.workload),
                      "kernel_sources_sha16": kernel_sources_sha(),
-                     "kernel": "k_step", "bytes_per_update": bpu, "peak_kind": peak_kind,
+                     "kernel": "k_step" if args.precision == "f64" else "k_even2/k_odd2", "bytes_per_update": bpu, "peak_kind": peak_kind,
                      "avg_kernel_us": avg_kernel_s * 1e6 if avg_kernel_s else None,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS if achieved else None,
                      "nominal_gbs": NOMINAL_HBM_GBS},
