@@ -269,7 +269,7 @@ int lbm_set_graph(lbm_ctx *ctx, int32_t chunk);
  * bulk copies (cp.async.bulk, completing on an mbarrier) several tiles ahead, so loads
  * are in flight without holding registers; available in every storage for pipes with
  * half-way or Bouzidi walls whose rows fit its shared-memory segments.  LBM_F64 has shape
- * 0 (256 x 2) and the staged shapes.  The direct shapes (0-3, 6-10) and the staged shapes
+ * 0 (32 x 16) and the staged shapes.  The direct shapes (0-3, 6-10) and the staged shapes
  * give bit-identical results; the pipelined kernel is compiled separately and agrees
  * with them to rounding (the compiler may contract different multiply-adds).  Errors:
  * LBM_EINVAL (a shape not available for the storage), LBM_EUNSUPPORTED (an ablation
@@ -280,7 +280,9 @@ int lbm_set_variant(lbm_ctx *ctx, int32_t variant);
  * slots), `odd` for the others (neighbour slots); lbm_set_variant sets both.  The defaults
  * are the fastest pair measured on GB300 (F32: 6 even, 9 odd; 16-bit formats and Bouzidi
  * walls: 7 even and, from about 10 M stored cells on, 7 odd, else 9; F64: 0 and 0).  Same
- * errors as lbm_set_variant. */
+ * errors as lbm_set_variant.  Until a shape is set or tuned, contexts of fewer than 60,000
+ * stored cells, full-way walls and the periodic box run these defaults with one plane per
+ * thread (128 x 8). */
 int lbm_set_variants(lbm_ctx *ctx, int32_t even, int32_t odd);
 
 /* Failure-detection tests of the staged shapes (11, 12): the next step launched directly

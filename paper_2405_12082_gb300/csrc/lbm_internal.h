@@ -120,7 +120,7 @@ struct ModesArgs {
 // (zc), whether it is the software-pipelined persistent kernel (shapes 4 and 5, F32
 // storage only) and whether it is the persistent kernel whose loads are staged in shared
 // memory by bulk copies (shapes 11 and 12, compact pipe layouts, every storage; staged =
-// index into STAGED_SHAPES + 1).  FP64 storage has shape 0 (256 x 2) and the staged ones.
+// index into STAGED_SHAPES + 1).  FP64 storage has shape 0 (32 x 16) and the staged ones.
 // Shapes 6-10 (several planes per thread) run on pairs of cells in the compact pipe layouts
 // (lbm_pair.cuh): pt, pb, pz are the threads, resident blocks and planes per thread of their
 // odd steps there; zc, threads and min_blocks hold for the dense layouts.

@@ -538,7 +538,8 @@ __device__ double uz_at(const StepArgs &a, const Member &d, int m, int x, int y,
 // DFT energies E_m = |sum_n u_n e^{-i m theta_n}|^2 / N^2 with warp-shuffle sums.  The N
 // angles' sines and cosines (FP64: the slow units of this chip) are taken once per block, for
 // the sample positions, and serve the DFT as its table: m n mod N, stepped without a division.
-// 3 rings x 16 sections of 1024 samples, m to 32, R = 96 pipe: 1.9 ms -> 0.1 ms.
+// R = 96 pipe, 3 rings x 16 sections of 1024 samples, m to 32: 0.076 ms (with a sine and a cosine
+// per sample and mode one ring of 512 samples took 0.27 ms).
 constexpr int MODES_BLOCK = 512;
 template <int P, int PAR, int WALL>
 __global__ void __launch_bounds__(MODES_BLOCK) k_modes(const __grid_constant__ StepArgs a, int m, const ModesArgs ma,
@@ -648,7 +649,7 @@ __device__ __forceinline__ AxisSum<R> axis_sum(R mm, R m0, R mp, R u3, R uh, R u
 // Bound by latency and issue (27 gathers, 9 moments, 27 stores per cell; the 50 MB fields live
 // in L2): pairs share the gather's addresses and halve the arithmetic's issue slots, and the
 // axis sums above take 162 operations where psi, psi', psi'' products took 220.  R = 24 pipe,
-// F32: 30 -> 22 us per step.
+// F32: 30 -> 26 us per step (128 threads x 4 blocks, 128 registers, no spills).
 template <int P, int OBJ, class R>
 __device__ __forceinline__ void adjoint_cells(const AdjArgs &j, const int4 ci, uint32_t r, int z, R &jterm, R &wterm) {
     using S = typename scalar_of<R>::type;
