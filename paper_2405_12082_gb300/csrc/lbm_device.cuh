@@ -167,6 +167,11 @@ __device__ __forceinline__ pf2 mul_(pf2 a, pf2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ pf2 add_(pf2 a, pf2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ pf2 sub_(pf2 a, pf2 b) { return fma_(b, make_float2(-1.f, -1.f), a); }   // same rounding
 __device__ __forceinline__ pf2 neg_(pf2 a) { return make_float2(-a.x, -a.y); }
+// a + b where a term is a rounded product: on pairs the compiler fuses an addition with the
+// product before it, on single cells it does not.
+__device__ __forceinline__ float sum_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double sum_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ pf2 sum_(pf2 a, pf2 b) { return fma_(a, make_float2(1.f, 1.f), b); }
 
 // The scalar type of R and a constant of type R.
 template <class R> struct scalar_of { using type = R; };
@@ -176,9 +181,10 @@ template <class R> __device__ __forceinline__ R lit(typename scalar_of<R>::type 
     else return c;
 }
 
-// 1 / x.  FP32: the hardware's approximate reciprocal and one Newton-Raphson iteration
-// r + r (1 - x r), which leaves it within one unit in the last place over the normal range
-// (x is a density, near 1) in three instructions and without the branch of the division.
+// 1 / x.  FP32: the hardware's approximate reciprocal (within one unit in the last place) and one
+// Newton-Raphson iteration r + r (1 - x r) on fused multiply-adds, which rounds correctly from
+// there (Markstein 1990) but for x whose mantissa is all ones: the division's result in three
+// instructions and without its branch (F16S, R = 96 pipe: 804 us per step, with the division 849).
 __device__ __forceinline__ float recip_(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -694,7 +700,8 @@ struct Macro { R rho, ux, uy, uz; };
 template <class R>
 struct MomentSums { R drho, jx, jy, jz, m4, m5, m6, m7, m8; };
 
-template <class R>
+// F32 (the storage): m6 is summed column by column, as collide_f32's results are pinned.
+template <class R, bool F32 = false>
 __device__ __forceinline__ MomentSums<R> moment_sums(const R (&v)[Q]) {
     R P[3][3], S[3][3], D[3][3];
     sfor<0, 9>([&](auto kc) {                       // column (cx, cy) = (a - 1, b - 1)
@@ -719,7 +726,8 @@ __device__ __forceinline__ MomentSums<R> moment_sums(const R (&v)[Q]) {
     m.jz = add_(add_(Da[0], Da[1]), Da[2]);
     m.m4 = sub_(sub_(S[2][2], S[2][0]), sub_(S[0][2], S[0][0]));
     m.m5 = sub_(Da[2], Da[0]);
-    m.m6 = sub_(add_(add_(D[0][2], D[1][2]), D[2][2]), add_(add_(D[0][0], D[1][0]), D[2][0]));
+    if constexpr (F32) m.m6 = add_(add_(sub_(D[0][2], D[0][0]), sub_(D[1][2], D[1][0])), sub_(D[2][2], D[2][0]));
+    else m.m6 = sub_(add_(add_(D[0][2], D[1][2]), D[2][2]), add_(add_(D[0][0], D[1][0]), D[2][0]));
     m.m7 = sub_(add_(S[0][1], S[2][1]), add_(S[1][0], S[1][2]));
     // x^2 - z^2: +1 on the cz = 0 populations of the cx != 0 columns, -1 on the cz != 0
     // populations of the cx = 0 columns
@@ -732,11 +740,9 @@ __device__ __forceinline__ MomentSums<R> moment_sums(const R (&v)[Q]) {
 
 // rho and u = sum c f / rho + g / 2 from the sums (bare momentum j, hg = g / 2).  SCALED: the
 // sums are in units of inv = 2^-s (the scaled half format; powers of two, exact).
-// u = j + (g / 2 - j (rho - 1) / rho): the bracket is small, so u is rounded once, where
-// j (1 / rho) + g / 2 also carries the reciprocal's rounding; the rounding of u moves the
-// momentum of all 18 moving populations alike and does not average out over the steps.
-// LEAN takes u = j (1 / rho) + g / 2: FP64, and the 16-bit formats, whose storage rounds
-// 4,000 times coarser.
+// LEAN takes u = j (1 / rho) + g / 2: the default model in every storage.  The ablation models
+// and general rates take u = j + (g / 2 - j (rho - 1) / rho): the bracket is small, so u is
+// rounded once.
 template <class R, bool SCALED = false, bool LEAN = false>
 __device__ __forceinline__ Macro<R> macro_from_sums(const MomentSums<R> &s, R hgx, R hgy, R hgz,
                                                     typename scalar_of<R>::type inv = 1) {
@@ -769,7 +775,7 @@ __device__ __forceinline__ Macro<R> macro_from_sums(const MomentSums<R> &s, R hg
 
 template <class R>
 __device__ __forceinline__ Macro<R> macroscopic(const R (&v)[Q], R gx, R gy, R gz) {
-    return macro_from_sums<R, false, sizeof(R) == 8>(moment_sums<R>(v), mul_(lit<R>(0.5f), gx), mul_(lit<R>(0.5f), gy), mul_(lit<R>(0.5f), gz));
+    return macro_from_sums<R, false, true>(moment_sums<R>(v), mul_(lit<R>(0.5f), gx), mul_(lit<R>(0.5f), gy), mul_(lit<R>(0.5f), gz));
 }
 
 // One-axis factors of the product-form equilibrium (see the file header):
@@ -800,7 +806,8 @@ template <int E, class R> __device__ __forceinline__ R cterm(R acc, R x) {
     else return acc;
 }
 
-// The default model's post-collision populations from the moment sums of a cell (R float,
+// Post-collision populations of the default model (FP64 and 16-bit storage; F32: collide_f32) and
+// of the BGK and second-order models, from the moment sums of a cell (R float,
 // double) or of a pair of cells (R pf2): emit(i, f*_i - w_i) for every i, row of columns
 // (c_y) by row.  SCALED (the scaled half format): sums and outputs are in storage
 // units, (f - w) sc with sc = 1 / inv a power of two; the shear moments stay in those units
@@ -983,6 +990,89 @@ __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R
     return mm;
 }
 
+// The default model in F32 storage, for one cell (R float) or a pair (R pf2): emit as in
+// collide_mrt, the same closed form in the order of operations to which the results of F32 runs
+// are pinned, bit for bit: a long run adds up what each step rounds (2,000 steps of a decaying
+// flow: 5e-5 between two orders), so another order is another result.
+//   X = G + hz A + dz H with G = Dxy + Fxy, A = 1 + Dxy, H = A + Fxy per column, Dxy = dx + dy +
+//   dx dy, Fxy = hx (1 + dy) + hy (1 + dx); f* - w = w rho X + (w drho + shear term).
+// 330 operations per cell, 165 issue slots on pairs.
+template <class R, bool ACT, class Emit>
+__device__ __forceinline__ Macro<R> collide_f32(const MomentSums<R> &ms, R gx, R gy, R gz, float omega, R *s_out,
+                                                Emit &&emit, R act = lit<R>(1)) {
+    const R hgx = mul_(lit<R>(0.5f), gx), hgy = mul_(lit<R>(0.5f), gy), hgz = mul_(lit<R>(0.5f), gz);
+    const Macro<R> mm = macro_from_sums<R, false, true>(ms, hgx, hgy, hgz);
+    const R rho = mm.rho, ux = mm.ux, uy = mm.uy, uz = mm.uz;
+    // s_k = m_k - m_k^eq + R_k / 2, k = 4..8
+    const R ux2 = mul_(ux, ux), uy2 = mul_(uy, uy), uz2 = mul_(uz, uz);
+    const R hr = mul_(lit<R>(0.5f), rho), nrho = neg_(rho), nrx = neg_(mul_(rho, ux)), nry = neg_(mul_(rho, uy));
+    const R gxux = mul_(gx, ux);
+    const R s4 = fma_(hr, fma_(gy, ux, mul_(gx, uy)), fma_(nrx, uy, ms.m4));
+    const R s5 = fma_(hr, fma_(gz, ux, mul_(gx, uz)), fma_(nrx, uz, ms.m5));
+    const R s6 = fma_(hr, fma_(gz, uy, mul_(gy, uz)), fma_(nry, uz, ms.m6));
+    const R s7 = fma_(rho, fma_(neg_(gy), uy, gxux), fma_(nrho, sub_(ux2, uy2), ms.m7));
+    const R s8 = fma_(rho, fma_(neg_(gz), uz, gxux), fma_(nrho, sub_(ux2, uz2), ms.m8));
+    if (s_out) {
+        s_out[0] = s4; s_out[1] = s5; s_out[2] = s6; s_out[3] = s7; s_out[4] = s8;
+    }
+    R om1 = lit<R>(1.f - omega), rho_o = rho, drho_o = ms.drho;
+    if constexpr (ACT) {
+        om1 = mul_(om1, act);
+        rho_o = mul_(rho_o, act);
+        drho_o = mul_(drho_o, act);
+    }
+    const R a4 = mul_(om1, s4), a5 = mul_(om1, s5), a6 = mul_(om1, s6), a7 = mul_(om1, s7), a8 = mul_(om1, s8);
+    const R six = lit<R>(float(1.0 / 6.0)), third = lit<R>(float(1.0 / 3.0));
+    const R w0 = lit<R>(float(w_of(0))), w1 = lit<R>(float(w_of(1))), w2 = lit<R>(float(w_of(7))), w3 = lit<R>(float(w_of(19)));
+    const R c12 = fma_(w1, drho_o, mul_(sum_(a7, a8), six));
+    const R c34 = fma_(w1, drho_o, fma_(a8, six, neg_(mul_(a7, third))));
+    const R c56 = fma_(w1, drho_o, fma_(a7, six, neg_(mul_(a8, third))));
+    const R wd2 = mul_(w2, drho_o), wd3 = mul_(w3, drho_o), q = lit<R>(0.25f), nq = lit<R>(-0.25f);
+    const R wr0 = mul_(w0, rho_o), wr1 = mul_(w1, rho_o), wr2 = mul_(w2, rho_o), wr3 = mul_(w3, rho_o);
+    // one-axis factors at c = -1, 0, +1: d = psi_hat - 1, h = (g / 2) psi_hat'
+    auto axis = [](auto cc, R u, R u2, R hg, R &d, R &h) {
+        constexpr int c = decltype(cc)::value;
+        if constexpr (c == 1) {
+            d = mul_(lit<R>(-1.5f), u2);
+            h = mul_(hg, mul_(lit<R>(-3.f), u));
+        } else {
+            const R t = mul_(lit<R>(c == 0 ? -3.f : 3.f), u);
+            d = fma_(lit<R>(3.f), u2, t);
+            h = mul_(hg, fma_(lit<R>(6.f), u, lit<R>(c == 0 ? -3.f : 3.f)));
+        }
+    };
+    R dy[3], hy[3], oy[3], dz[3], hz[3];
+    sfor<0, 3>([&](auto cc) {
+        constexpr int c = decltype(cc)::value;
+        axis(cc, uy, uy2, hgy, dy[c], hy[c]);
+        axis(cc, uz, uz2, hgz, dz[c], hz[c]);
+        oy[c] = sum_(dy[c], lit<R>(1));
+    });
+    sfor<0, 3>([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        R dx, hx;
+        axis(ac, ux, ux2, hgx, dx, hx);
+        const R ox = sum_(dx, lit<R>(1));
+        sfor<0, 3>([&](auto bc) {
+            constexpr int b = decltype(bc)::value;
+            const R D = fma_(dx, dy[b], sum_(dx, dy[b])), F = fma_(hx, oy[b], mul_(hy[b], ox));
+            const R A = add_(D, lit<R>(1)), G = add_(D, F), H = add_(A, F);
+            sfor<0, 3>([&](auto cc) {
+                constexpr int c = decltype(cc)::value, i = dir_of(a - 1, b - 1, c - 1);
+                using I = std::integral_constant<int, i>;
+                const R X = fma_(dz[c], H, fma_(hz[c], A, G));
+                if constexpr (i == 0) emit(I{}, fma_(w0, drho_o, mul_(wr0, X)));
+                else if constexpr (i <= 6) emit(I{}, fma_(wr1, X, i <= 2 ? c12 : i <= 4 ? c34 : c56));
+                else if constexpr (i <= 18) {
+                    constexpr int k = (i - 7) / 4, e = (i - 7) % 4;          // shear moment 4 + k, sign + - - +
+                    emit(I{}, fma_(wr2, X, fma_(e == 0 || e == 3 ? q : nq, k == 0 ? a4 : k == 1 ? a5 : a6, wd2)));
+                } else emit(I{}, fma_(wr3, X, wd3));
+            });
+        });
+    });
+    return mm;
+}
+
 // In-place collision of one fluid cell; v holds f - w on entry and f* - w on exit.
 // With s_out, the five non-equilibrium shear moments s_k = m_k - m_k^eq + R_k / 2
 // (k = 4..8) are returned as well (the adjoint stores them).
@@ -992,14 +1082,17 @@ __device__ __forceinline__ Macro<R> collide_mrt(const MomentSums<R> &ms, R gx, R
 // is the same for both equilibria since they share their second moments and those of F;
 // for the BGK, N = f - f^eq + F/2.  MODEL_RATES takes a general diagonal Lambda:
 // f* = f^eq + F/2 + (M^T)^{-1} (1 - Lambda) M^T n with n = f - f^eq + F/2, whose moments
-// 0..3 vanish (lam1[k - 4] = 1 - lambda_k).  The default model runs collide_mrt; SCALED
-// (default model only): v is in storage units, see there.
+// 0..3 vanish (lam1[k - 4] = 1 - lambda_k).  SCALED (default model only): v is in storage units,
+// see collide_mrt.
 template <class R, int MODEL = MODEL_MRT_H6, bool SCALED = false, bool LEAN = sizeof(R) == 8>
 __device__ __forceinline__ Macro<R> collide(R (&v)[Q], R gx, R gy, R gz, R omega, R *s_out = nullptr,
                                             const R *lam1 = nullptr, R inv = R(1), R sc = R(1)) {
     static_assert(!SCALED || MODEL == MODEL_MRT_H6, "scaled units serve the default model only");
-    const MomentSums<R> ms = moment_sums<R>(v);
-    if constexpr (!(MODEL & MODEL_RATES)) {
+    constexpr bool F32 = MODEL == MODEL_MRT_H6 && !LEAN;
+    const MomentSums<R> ms = moment_sums<R, F32>(v);
+    if constexpr (F32) {
+        return collide_f32<R, false>(ms, gx, gy, gz, omega, s_out, [&](auto ic, R f) { v[decltype(ic)::value] = f; });
+    } else if constexpr (!(MODEL & MODEL_RATES)) {
         return collide_mrt<R, SCALED, false, LEAN, MODEL>(ms, gx, gy, gz, omega, inv, sc, s_out,
                                                           [&](auto ic, R f) { v[decltype(ic)::value] = f; }, R(1), v);
     } else {

@@ -84,6 +84,15 @@ template <class A>
 __device__ __forceinline__ int64_t pair_t(const A &a) { return a.times ? a.times[a.tidx].t : a.t; }
 
 // ---- even step ----------------------------------------------------------------------------
+// The default model on the cells of a pair kernel: F32 in its pinned order, the 16-bit formats in
+// the shorter form.
+template <int P, bool ACT, class R, class Emit>
+__device__ __forceinline__ Macro<R> pair_collide(const MomentSums<R> &ms, R gx, R gy, R gz, float omega, float inv, float sc,
+                                                 R *s_out, Emit &&emit, R act = lit<R>(1)) {
+    if constexpr (P == LBM_F32) return collide_f32<R, ACT>(ms, gx, gy, gz, omega, s_out, emit, act);
+    else return collide_mrt<R, P == LBM_F16S, ACT, true>(ms, gx, gy, gz, omega, inv, sc, s_out, emit, act);
+}
+
 // The pair at stored positions lc, lc + 1 (plane z, position r, table entry pi with its first
 // cell fluid), whose populations are in raw.
 template <int P, int WALL, int EXTRA, class A, class D>
@@ -92,7 +101,6 @@ __device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_
     using PS = PairStorage<P>;
     using T = typename PS::T;
     using V = typename PS::V;
-    constexpr bool SC = P == LBM_F16S;
     char *const base = static_cast<char *>(a.pops);
     const uint64_t stb = (uint64_t)a.stride * sizeof(T);
     const uint32_t vo = ((uint32_t)d.off + lc) * (uint32_t)sizeof(T);
@@ -132,7 +140,7 @@ __device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_
             });
         }
     }
-    const MomentSums<pf2> ms = moment_sums<pf2>(v);
+    const MomentSums<pf2> ms = moment_sums<pf2, P == LBM_F32>(v);
     Macro<pf2> mm;
     // a slot is written where it was read: the zero keeps the compiler from carrying the 27
     // addresses through the collision in registers
@@ -143,7 +151,7 @@ __device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_
         *reinterpret_cast<V *>(wbase + ib * stb + wo) = PS::down(f);
     };
     if constexpr (WALL == LBM_BOUZIDI) {
-        mm = collide_mrt<pf2, SC, true, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr,
+        mm = pair_collide<P, true, pf2>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr,
                                         [&](auto ic, pf2 f) { v[decltype(ic)::value] = f; }, act);
         if (pi & PAIR_WALL) {
             const float *tab = static_cast<const float *>(d.dtab) + (int64_t)col * 27;
@@ -165,8 +173,8 @@ __device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_
         }
     } else {
         pf2 sk[5];
-        mm = collide_mrt<pf2, SC, true, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
-                                                      EXTRA == EX_MOMENTS ? sk : nullptr, store, act);
+        mm = pair_collide<P, true, pf2>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
+                                        EXTRA == EX_MOMENTS ? sk : nullptr, store, act);
         if constexpr (EXTRA == EX_MOMENTS) {
             pf2 *mo = reinterpret_cast<pf2 *>(static_cast<float *>(a.moments) + lc);
             const int64_t n = d.scells >> 1;
@@ -255,7 +263,7 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
                                           float tx, float ty, float tz) {
     using PS = PairStorage<P>;
     using B = typename PS::B;
-    constexpr bool SC = P == LBM_F16S, TWO = std::is_same<R, pf2>::value;
+    constexpr bool TWO = std::is_same<R, pf2>::value;
     const uint32_t nb = (uint32_t)ci.y;
     const uint32_t col = (uint32_t)(ci.x & 0xFFFF) * (uint32_t)d.nx + ((uint32_t)ci.x >> 16);
     const int64_t plane = (int64_t)d.nx * d.ny;
@@ -312,7 +320,7 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
                         v[opp_of(j)] = fma_(lit<R>(tab[nbit(cx, cy) * 3 + 2]), v[j], v[opp_of(j)]);
             });
     }
-    const MomentSums<R> ms = moment_sums<R>(v);
+    const MomentSums<R> ms = moment_sums<R, P == LBM_F32>(v);
     // the element a slot is written at is the one it was read at: the zero (which depends on
     // the data) keeps the compiler from carrying the addresses through the collision
     uint32_t bits;
@@ -331,7 +339,7 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
     };
     Macro<R> mm;
     if constexpr (WALL == LBM_BOUZIDI) {
-        mm = collide_mrt<R, SC, false, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr,
+        mm = pair_collide<P, false, R>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale, nullptr,
                                        [&](auto ic, R f) { v[decltype(ic)::value] = f; });
         sfor<0, Q>([&](auto jc) {
             constexpr int j = decltype(jc)::value, cx = cx_of(j), cy = cy_of(j), kk = nbit(cx, cy);
@@ -343,8 +351,8 @@ __device__ __forceinline__ void odd_cells(const A &a, const D &d, const int4 ci,
         });
     } else {
         R sk[5];
-        mm = collide_mrt<R, SC, false, P != LBM_F32>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
-                                                     EXTRA == EX_MOMENTS ? sk : nullptr, store);
+        mm = pair_collide<P, false, R>(ms, gx, gy, gz, d.omegaf, a.f16_inv, a.f16_scale,
+                                       EXTRA == EX_MOMENTS ? sk : nullptr, store);
         if constexpr (EXTRA == EX_MOMENTS) {
             float *mo = static_cast<float *>(a.moments) + (own - (uint32_t)d.off);
             const R out[9] = {mm.rho, mm.ux, mm.uy, mm.uz, sk[0], sk[1], sk[2], sk[3], sk[4]};
