@@ -249,7 +249,8 @@ int lbm_step(lbm_ctx *ctx, int64_t n);
  * steps (even, 2..4096; 0 = direct launches) whenever at least `chunk` steps remain
  * and t is even (and a multiple of the statistics interval when statistics are on);
  * the rest run as direct launches.  The graph is captured once per launch shape and
- * statistics setting; every node reads its step index and trigger phase from a
+ * statistics setting, and again after lbm_set_force or lbm_set_relax changed a member
+ * whose steps run on pairs of cells (lbm_set_variant); every node reads its step index and trigger phase from a
  * device table that the host refreshes before each replay, so results are
  * bit-identical to direct launches.  Allocates the tables (device + pinned host). */
 int lbm_set_graph(lbm_ctx *ctx, int32_t chunk);

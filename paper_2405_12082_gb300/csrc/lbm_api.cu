@@ -65,6 +65,7 @@ struct lbm_ctx {
     int32_t graph_chunk = 0;
     cudaGraphExec_t gexec = nullptr;
     int gexec_variant = -1, gexec_variant_odd = -1, gexec_stats_every = -1;
+    bool gexec_by_value = false;     // its nodes carry the members in their parameters (pair kernels)
     lbm::StepTime *d_times = nullptr;        // [graph_chunk] device table read by the graph
     lbm::StepTime *h_times[2] = {nullptr, nullptr};   // pinned staging, double-buffered
     cudaEvent_t h_done[2] = {nullptr, nullptr};
@@ -394,6 +395,8 @@ void fill_force(Member &d, const lbm_force *f) {
     d.gz_field = f ? f->gz_field : nullptr;
 }
 
+int upload_members(lbm_ctx *c);
+
 int check_relax(lbm_ctx *c, const lbm_relax *r) {
     if (!(r->omega > 0.0 && r->omega < 2.0)) return set_err(c, LBM_EINVAL, "omega must be in (0, 2)");
     if (r->rates)
@@ -414,6 +417,15 @@ void fill_lambda(Member &d, const double *rates, int model_bits) {
 }
 
 void drop_graph(lbm_ctx *c);
+
+// Hands a changed member m (`before`: what it was) to the kernels: the device table, which most
+// steps read, and a captured graph of pair kernels, which hold its fields -- force, omega, the
+// address of the force field -- as of their capture, by a new capture at the next replay.
+int publish_member(lbm_ctx *c, int m, const Member &before) {
+    const int rc = upload_members(c);
+    if (c->gexec_by_value && std::memcmp(&before, &c->hm[m], sizeof before) != 0) drop_graph(c);
+    return rc;
+}
 
 // Recomputes every member's relaxation table and the step kernel's collision code; a new
 // code returns the launch shape to the default and drops a captured graph.
@@ -921,6 +933,7 @@ int lbm_set_relax(lbm_ctx *c, const lbm_relax *r) {
     int rc = check_relax(c, r);
     if (rc) return rc;
     const int m = c->sel;
+    const Member before = c->hm[m];
     const bool had = c->has_rates[m];
     const double omega0 = c->hm[m].omega;
     const std::array<double, 27> rates0 = c->rates[m];
@@ -937,18 +950,19 @@ int lbm_set_relax(lbm_ctx *c, const lbm_relax *r) {
         update_collision(c);
         return rc;
     }
-    return upload_members(c);
+    return publish_member(c, m, before);
 }
 
 int lbm_set_force(lbm_ctx *c, const lbm_force *f) {
     if (!c) return LBM_EINVAL;
     int rc = check_force(c, f);
     if (rc) return rc;
+    const Member before = c->hm[c->sel];
     fill_force(c->hm[c->sel], f);
     lbm_force fz;
     std::memset(&fz, 0, sizeof fz);
     c->forces[c->sel] = f ? *f : fz;
-    rc = upload_members(c);
+    rc = publish_member(c, c->sel, before);
     if (rc) return rc;
     return fill_force_tables(c, c->sel);
 }
@@ -1062,6 +1076,7 @@ int step_direct(lbm_ctx *c, bool overlap = false) {
 void drop_graph(lbm_ctx *c) {
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
+    c->gexec_by_value = false;
     c->gexec_variant = -1;
     c->gexec_variant_odd = -1;
     c->gexec_stats_every = -1;
@@ -1113,6 +1128,7 @@ int build_graph(lbm_ctx *c) {
         c->gexec = nullptr;
         return cuda_err(c, e, "cudaGraphInstantiate");
     }
+    c->gexec_by_value = ap[0].pairs || ap[1].pairs;
     c->gexec_variant = c->variant;
     c->gexec_variant_odd = c->variant_odd;
     c->gexec_stats_every = every;
