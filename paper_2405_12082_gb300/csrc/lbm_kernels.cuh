@@ -163,7 +163,9 @@ __device__ __forceinline__ TileCell tile_cell(const StepArgs &a, int tile) {
         c.m = find_member(a, tile);
         const Member &d = a.members[c.m];
         const uint32_t local = (uint32_t)(tile - a.block0[c.m]) * BS + threadIdx.x;
-        if (local < (uint32_t)d.scells) c.active = cell_from_storage(d, local, c.p);
+        // the grid covers the fluid columns of a dense pipe (make_args), else the stored cells
+        if (d.fluidcol != nullptr) c.active = cell_from_work(d, local, 1, c.p);
+        else if (local < (uint32_t)d.scells) c.active = cell_from_storage(d, local, c.p);
     }
     return c;
 }
