@@ -1518,7 +1518,7 @@ int lbm_modes(lbm_ctx *c, const lbm_modes_cfg *cfg, double *E) {
     if (d.geometry != LBM_PIPE) return set_err(c, LBM_EINVAL, "modes need a pipe");
     if (cfg->n_sections < 1 || cfg->n_sections > d.nz) return set_err(c, LBM_EINVAL, "n_sections must be in 1..nz");
     if (cfg->n_rings < 1 || cfg->n_rings > 16) return set_err(c, LBM_EINVAL, "n_rings must be in 1..16");
-    if (cfg->n_theta < 8 || cfg->n_theta > 4096) return set_err(c, LBM_EINVAL, "n_theta must be in 8..4096");
+    if (cfg->n_theta < 8 || cfg->n_theta > lbm::MODES_MAX_THETA) return set_err(c, LBM_EINVAL, "n_theta must be in 8..4096");
     if (cfg->n_modes < 0 || cfg->n_modes >= cfg->n_theta) return set_err(c, LBM_EINVAL, "n_modes must be in 0..n_theta-1");
     lbm::ModesArgs ma;
     std::memset(&ma, 0, sizeof ma);

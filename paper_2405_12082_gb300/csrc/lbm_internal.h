@@ -110,6 +110,7 @@ cudaError_t launch_step_kernel(void (*kern)(const A), int blocks, int threads, b
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
+constexpr int MODES_MAX_THETA = 4096;        // samples of a ring (lbm_modes)
 struct ModesArgs {
     int32_t n_sections, n_rings, n_theta, n_modes;
     double r_over_R[16];

@@ -1278,7 +1278,10 @@ cudaError_t launch_modes(int wall, int parity, const StepArgs &a, const Member &
     const size_t shm = 3 * (size_t)ma.n_theta * sizeof(double);
     LBM_DISPATCH_WP(wall, parity, {
         if (shm > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k_modes<P, PA, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+            // the limit is the kernel's, which every context and thread shares: always the largest
+            // ring's, so that no call lowers it between another's limit and launch
+            cudaError_t e = cudaFuncSetAttribute(k_modes<P, PA, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 3 * MODES_MAX_THETA * (int)sizeof(double));
             if (e != cudaSuccess) return e;
         }
         k_modes<P, PA, W><<<nblk, MODES_BLOCK, shm, s>>>(a, m, ma, E);
