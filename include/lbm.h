@@ -146,8 +146,10 @@ typedef struct {
     int32_t n_members;
     int32_t precision;
     int64_t launches;       /* kernels this context has launched so far              */
-    int32_t variant;        /* launch shape of the step kernel (lbm_set_variant)     */
-    int32_t step_threads;   /* threads per block of that shape                       */
+    int32_t variant;        /* launch shape of the step kernel (lbm_set_variant);    */
+                            /* until one is set the defaults 6, 7 and 9 may run one  */
+                            /* plane per thread (lbm_set_variants)                   */
+    int32_t step_threads;   /* threads per block of the even steps as they run       */
     int32_t n_variants;     /* launch shapes available for this precision            */
     int32_t graph_chunk;    /* steps per captured graph, 0 = direct launches         */
     int32_t variant_odd;    /* launch shape of the odd steps (variant: the even ones) */
@@ -262,8 +264,9 @@ int lbm_set_graph(lbm_ctx *ctx, int32_t chunk);
  * computes the current one); 6-10 = several planes per thread: 128 x 8 with 2
  * and with 4 planes, 256 x 4, 128 x 7 and 128 x 6 with 2 (full-way walls, periodic box); on
  * pipes with half-way or Bouzidi walls in LBM_F32 and the 16-bit formats these run on pairs
- * of cells with the paired FP32 instructions, even steps 128 x 5 on neighbours in x, odd
- * steps on neighbours in z: 6 = 256 x 2 and 9 = 128 x 4 with 2 planes per thread, 7 = 128 x 4
+ * of cells with the paired FP32 instructions, even steps on neighbours in x (128 x 5 with a
+ * pair per thread; half-way walls in the 16-bit formats 128 x 4 with two), odd steps on
+ * neighbours in z: 6 = 256 x 2 and 9 = 128 x 4 with 2 planes per thread, 7 = 128 x 4
  * and 8 = 64 x 8 with 4, 10 = 128 x 4 with 8; 11 and 12 = the staged persistent kernel (512
  * threads with 3 tiles in flight, one CTA per SM; 256 threads, 3 tiles, two CTAs per SM): a
  * tile is a group of whole fluid rows of one plane, whose populations the kernel copies with

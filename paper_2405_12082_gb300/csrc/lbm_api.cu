@@ -538,6 +538,28 @@ bool pairs_of(const lbm_ctx *c) {
     return true;
 }
 
+// What runs when launch shape v is due: of the shapes of several planes per thread, pairs of cells
+// where the context has them (unless it is small and left to the default), else one plane per
+// thread for Bouzidi walls and wherever no shape was set -- without pairs that is the faster one
+// (full-way R = 48 pipe, F32: 147.4 us per step against 149 to 154), also where there are too few
+// cells to give a thread several.
+struct ShapeRun {
+    bool pairs, single;
+    int threads, zc;         // of a block (pairs: of the even steps); planes per thread
+};
+ShapeRun shape_run(const lbm_ctx *c, int v) {
+    ShapeRun r = {false, false, lbm::step_threads(c->precision, v), lbm::step_zc(c->precision, v)};
+    if (r.zc == 1) return r;
+    r.pairs = (c->shape_set || c->stride >= PAIRS_MIN_CELLS) && pairs_of(c);
+    r.single = !r.pairs && (c->wall == LBM_BOUZIDI || !c->shape_set);
+    if (r.pairs) r.threads = lbm::EVEN2_THREADS;
+    if (r.single) {
+        r.threads = lbm::SINGLE_THREADS;
+        r.zc = 1;
+    }
+    return r;
+}
+
 StepArgs make_args(const lbm_ctx *c, int64_t t) {
     StepArgs a;
     std::memset(&a, 0, sizeof a);
@@ -552,7 +574,9 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
     a.dstride = c->dense_total;
     a.collision = c->collision;
     const int v = variant_at(c, t);
-    int bs = lbm::step_threads(c->precision, v), zc = lbm::step_zc(c->precision, v);
+    const ShapeRun run = shape_run(c, v);
+    const bool pairs = run.pairs;
+    const int bs = run.threads, zc = run.zc;
     const int sk = lbm::staged_of(v);
     a.err = c->flags;
     a.skip_tile = -1;
@@ -561,15 +585,8 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         a.sg_sel = sk;
     }
     int64_t blk = 0;
-    const bool pairs = zc > 1 && (c->shape_set || c->stride >= PAIRS_MIN_CELLS) && pairs_of(c);
     a.pairs = pairs;
-    // without pairs one plane per thread is the faster shape (full-way R = 48 pipe, F32: 147.4 us
-    // per step against 149 to 154), also where there are too few cells to give a thread several
-    if (zc > 1 && !pairs && (c->wall == LBM_BOUZIDI || !c->shape_set)) {
-        bs = lbm::SINGLE_THREADS;
-        zc = 1;
-        a.single = 1;
-    }
+    a.single = run.single;
     for (size_t m = 0; m < c->hm.size(); ++m) {
         const Member &d = c->hm[m];
         a.st[m] = (d.trig && t < d.t_end) ? std::sin(2.0 * M_PI * (double)t / d.period) : 0.0;
@@ -578,7 +595,7 @@ StepArgs make_args(const lbm_ctx *c, int64_t t) {
         if (sk >= 0) {
             blk += (int64_t)d.nsg[sk] * d.nz;        // staged: one tile per (plane, row group)
         } else if (pairs && (t & 1) == 0) {
-            blk += ceil_div(d.scells / (2 * lbm::even_pairs(c->precision, c->wall)), 128);
+            blk += ceil_div(d.scells / (2 * lbm::even_pairs(c->precision, c->wall)), bs);
         } else if (pairs) {
             blk += ceil_div(d.Ps, lbm::STEP_SHAPES[v].pt) *
                    (lbm::odd_single_planes(d.nz) + lbm::odd_pair_groups(d.nz, lbm::STEP_SHAPES[v].pz));
@@ -922,7 +939,7 @@ int lbm_get_info(lbm_ctx *c, lbm_info *info) {
     info->launches = c->launches;
     info->variant = c->variant;
     info->variant_odd = c->variant_odd;
-    info->step_threads = lbm::step_threads(c->precision, c->variant);
+    info->step_threads = shape_run(c, c->variant).threads;
     info->n_variants = lbm::step_variants(c->precision);
     info->graph_chunk = c->graph_chunk;
     return LBM_OK;

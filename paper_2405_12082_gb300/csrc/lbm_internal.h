@@ -67,6 +67,7 @@ struct PairArgsMany : PairArgsBase {
 // 0.897, 6: 0.963 / 0.876).
 // The 16-bit formats' two pairs per thread take 128 registers (4 blocks).
 constexpr int even_pairs(int precision, int wall) { return precision == LBM_F32 || wall == LBM_BOUZIDI ? 1 : 2; }
+constexpr int EVEN2_THREADS = 128;
 template <int P, int WALL> constexpr int EVEN2_BLOCKS = even_pairs(P, WALL) == 1 ? 5 : 4;
 // Planes the odd pair kernel takes singly (0, nz - 1 and, for odd nz > 2, nz - 2), and its plane
 // groups of zc planes (the pairs 1 .. nz - 2) after them.
@@ -139,8 +140,8 @@ constexpr StepShape STEP_SHAPES[13] = {{256, 4, 1, 0, 0, 0, 0, 0},    {256, 3, 1
 // FP64 steps are bound by the FP64 units of each SM: blocks of one warp spread a small context
 // evenly over the SMs.
 constexpr StepShape STEP_SHAPE_F64 = {32, 16, 1, 0, 0, 0, 0, 0};
-// Threads per block where a shape of several planes per thread runs one (see make_args).
-constexpr int SINGLE_THREADS = 128;
+// Where a shape of several planes per thread runs one (see shape_run): shape 2.
+constexpr int SINGLE_VARIANT = 2, SINGLE_THREADS = STEP_SHAPES[SINGLE_VARIANT].threads;
 constexpr int N_STEP_SHAPES = 13;
 // Staged shapes: threads per CTA (one producer warp, the rest consume), pipeline stages
 // (tiles in flight per CTA), CTAs per SM and consumer groups (tiles worked on at once).

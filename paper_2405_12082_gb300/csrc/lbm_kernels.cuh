@@ -1015,8 +1015,8 @@ cudaError_t launch_pair_args(int parity, bool stats, int blocks, bool overlap, c
     cudaError_t e = cudaSuccess;
     constexpr StepShape S = STEP_SHAPES[V];
     if (parity == 0) {
-        if (stats) e = launch_step_kernel<A>(k_even2<P, WALL, EX_STATS, 128, EVEN2_BLOCKS<P, WALL>, A>, blocks, 128, overlap, a, s);
-        else e = launch_step_kernel<A>(k_even2<P, WALL, EX_NONE, 128, EVEN2_BLOCKS<P, WALL>, A>, blocks, 128, overlap, a, s);
+        if (stats) e = launch_step_kernel<A>(k_even2<P, WALL, EX_STATS, EVEN2_THREADS, EVEN2_BLOCKS<P, WALL>, A>, blocks, EVEN2_THREADS, overlap, a, s);
+        else e = launch_step_kernel<A>(k_even2<P, WALL, EX_NONE, EVEN2_THREADS, EVEN2_BLOCKS<P, WALL>, A>, blocks, EVEN2_THREADS, overlap, a, s);
     } else {
         if (stats) e = launch_step_kernel<A>(k_odd2<P, WALL, EX_STATS, S.pt, S.pb, S.pz, A>, blocks, S.pt, overlap, a, s);
         else e = launch_step_kernel<A>(k_odd2<P, WALL, EX_NONE, S.pt, S.pb, S.pz, A>, blocks, S.pt, overlap, a, s);
@@ -1073,7 +1073,7 @@ template <int P, int V>
 cudaError_t launch_planes(int wall, int parity, bool stats, const StepArgs &a, const Member *hm, cudaStream_t s) {
     if (a.pairs) return launch_pair<P, V>(wall, parity, stats, a, hm, s);
     constexpr StepShape S = STEP_SHAPES[V];
-    if (a.single) return launch_step_shape<P, SINGLE_THREADS, 1024 / SINGLE_THREADS>(wall, parity, stats, a, s);
+    if (a.single) return launch_step_shape<P, SINGLE_THREADS, STEP_SHAPES[SINGLE_VARIANT].min_blocks>(wall, parity, stats, a, s);
     const bool full = wall == LBM_FULLWAY;
     cudaError_t e = cudaSuccess;
     auto go = [&](auto pa, auto w) {
@@ -1132,7 +1132,7 @@ cudaError_t launch_step_moments(int parity, const StepArgs &a, const Member *hm,
             constexpr StepShape S = STEP_SHAPES[MOM_VARIANT_PAIRS];
             fill_pair_one<MOM_VARIANT_PAIRS>(o, a, hm);
             if (parity == 0)
-                return launch_step_kernel<PairArgsOne>(k_even2<P, LBM_HALFWAY, EX_MOMENTS, 128, EVEN2_BLOCKS<P, LBM_HALFWAY>, PairArgsOne>, a.nblocks_total, 128, a.overlap, o, s);
+                return launch_step_kernel<PairArgsOne>(k_even2<P, LBM_HALFWAY, EX_MOMENTS, EVEN2_THREADS, EVEN2_BLOCKS<P, LBM_HALFWAY>, PairArgsOne>, a.nblocks_total, EVEN2_THREADS, a.overlap, o, s);
             return launch_step_kernel<PairArgsOne>(k_odd2<P, LBM_HALFWAY, EX_MOMENTS, S.pt, S.pb, S.pz, PairArgsOne>, a.nblocks_total, S.pt, a.overlap, o, s);
         }
     }
