@@ -299,11 +299,13 @@ int lbm_set_variants(lbm_ctx *ctx, int32_t even, int32_t odd);
  * LBM_EUNSUPPORTED (the current shape is not staged). */
 int lbm_test_expire_wait(lbm_ctx *ctx, int32_t tile);
 
-/* Project autotuner for the launch shapes: times `steps` steps (2..10000) of every
- * shape on the context's own problem, the even and the odd steps separately, restores
- * the populations, t and statistics afterwards, selects the fastest shape for each parity
- * (lbm_set_variants) and returns the even one in *variant (lbm_get_info reports both) with
- * the mean time per step of the chosen pair (microseconds).  Synchronises; allocates one
+/* Project autotuner for the launch shapes: times `steps` steps (2..10000) on the
+ * context's own problem as lbm_step runs them (replays where lbm_set_graph's chunk fits
+ * into `steps`), for every shape at even t beside the present odd one, then for every
+ * shape at odd t beside the even one chosen; restores the populations, t and statistics
+ * afterwards, selects the fastest shape for each parity (lbm_set_variants) and returns the
+ * even one in *variant (lbm_get_info reports both) with the mean time per step of the
+ * chosen pair (microseconds).  Synchronises; allocates one
  * temporary copy of the populations. */
 int lbm_autotune(lbm_ctx *ctx, int32_t steps, int32_t *variant, double *best_us);
 
