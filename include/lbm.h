@@ -347,8 +347,9 @@ int lbm_set_raw(lbm_ctx *ctx, const void *buf, size_t bytes);
 int lbm_save(lbm_ctx *ctx, const char *path);
 int lbm_load(lbm_ctx *ctx, const char *path);
 
-/* Sum over fluid cells of the selected member, in FP64: out[0] = sum (rho - 1),
- * out[1..3] = sum of momentum sum_i c_i f_i, out[4] = number of cells with a
+/* Sum over fluid cells of the selected member, in FP64 (FP32 and 16-bit populations: to
+ * within the rounding of FP64 sums, in pairs of floats that lose nothing): out[0] = sum
+ * (rho - 1), out[1..3] = sum of momentum sum_i c_i f_i, out[4] = number of cells with a
  * non-finite population.  out is host memory; the call synchronises. */
 int lbm_reduce(lbm_ctx *ctx, double *out);
 

@@ -436,18 +436,24 @@ __device__ __forceinline__ void block_sum(double (&x)[NV], double *sh /* [NV][32
 
 // FP64 adds are what a sum of FP32 populations costs here (two lanes per SM and cycle: 81 adds
 // and 27 conversions per cell took 10 ms on the R = 96 pipe, against 0.55 ms for reading it).
-// So every thread keeps each population's sum over eight cells as an unevaluated pair hi + lo of
-// floats -- Knuth's two-sum: hi + x = s + e exactly, e collected in lo, about 48 bits -- and
-// only the pairs of eight cells enter FP64, through the z-triplets of moment_sums: 17 FP64
-// operations per cell.  A pair's rounding stays below that of the FP64 sum of a thread's
-// hundred cells it joins.  Cells with a value too large for FP32 sums (or not finite) are
-// added in FP64 one by one.
-constexpr int REDUCE_CELLS = 8;
+// So every thread keeps each population's sum over its cells as an unevaluated pair hi + lo of
+// floats -- Knuth's two-sum: hi + x = s + e exactly -- where e joins lo by another two-sum, whose
+// error (2^-48 of the magnitudes and less) goes to the thread's four sums r: nothing is lost but
+// the rounding of r, and a thread's 27 pairs enter FP64 once, through the z-triplets of
+// moment_sums.  (With lo's rounding dropped the pairs had to enter FP64 every eight cells and still
+// lost up to 2^-45: fields, rings and sums of the R = 96 pipe 2,215 us, now 1,878.)  Cells with a
+// value too large for FP32 sums (or not finite) are added in FP64.
 __device__ __forceinline__ void add_sums(double (&acc)[5], const MomentSums<double> &m) {
     acc[0] += m.drho;
     acc[1] += m.jx;
     acc[2] += m.jy;
     acc[3] += m.jz;
+}
+// a + b = s + e exactly; returns s.
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
 }
 template <int P, int PAR, int WALL>
 __global__ void __launch_bounds__(REDUCE_BLOCK, 2) k_reduce(const __grid_constant__ StepArgs a, int m,
@@ -456,20 +462,10 @@ __global__ void __launch_bounds__(REDUCE_BLOCK, 2) k_reduce(const __grid_constan
     __shared__ double sh[5 * 32];
     const Member &d = a.members[m];
     double acc[5] = {0, 0, 0, 0, 0};
-    float hi[Q], lo[Q];
+    float hi[Q], lo[Q], r[4] = {0.f, 0.f, 0.f, 0.f};      // r: mass, momentum
 #pragma unroll
     for (int i = 0; i < Q; ++i) hi[i] = lo[i] = 0.f;
-    auto flush = [&]() {
-        double x[Q];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            x[i] = __dadd_rn((double)hi[i], (double)lo[i]);
-            hi[i] = lo[i] = 0.f;
-        }
-        add_sums(acc, moment_sums<double>(x));
-    };
     const int64_t work = (int64_t)d.Pw * d.nz;
-    int held = 0;                          // counted per pass, not per cell: all lanes flush together
     for (int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; local < work;
          local += (int64_t)gridDim.x * blockDim.x) {
         CellPos p;
@@ -480,30 +476,50 @@ __global__ void __launch_bounds__(REDUCE_BLOCK, 2) k_reduce(const __grid_constan
 #pragma unroll
             for (int i = 0; i < Q; ++i) wide |= !(fabs(v[i]) < R(1e30));
             if (sizeof(R) == 8 || wide) {
-                double x[Q];
                 bool bad = false;
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    x[i] = (double)v[i];
-                    bad |= !isfinite(x[i]);
-                }
-                add_sums(acc, moment_sums<double>(x));
+                for (int i = 0; i < Q; ++i) bad |= !isfinite(v[i]);
                 acc[4] += bad ? 1.0 : 0.0;
-            } else if constexpr (sizeof(R) == 4) {
+            }
+            if constexpr (sizeof(R) == 8) {
+                add_sums(acc, moment_sums<double>(v));
+            } else if (wide) {
+                sfor<0, Q>([&](auto ic) {
+                    constexpr int i = decltype(ic)::value, c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+                    const double x = (double)v[i];
+                    acc[0] += x;
+                    if constexpr (c[0] != 0) acc[1] += c[0] * x;
+                    if constexpr (c[1] != 0) acc[2] += c[1] * x;
+                    if constexpr (c[2] != 0) acc[3] += c[2] * x;
+                });
+            } else {
+                sfor<0, 9>([&](auto kc) {                       // the z-triplet of column (cx, cy)
+                    constexpr int cx = decltype(kc)::value % 3 - 1, cy = decltype(kc)::value / 3 - 1;
+                    float q[3];
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    const float s = __fadd_rn(hi[i], v[i]), t = __fsub_rn(s, hi[i]);
-                    lo[i] = __fadd_rn(lo[i], __fadd_rn(__fsub_rn(hi[i], __fsub_rn(s, t)), __fsub_rn(v[i], t)));
-                    hi[i] = s;
-                }
+                    for (int z = 0; z < 3; ++z) {
+                        const int i = dir_of(cx, cy, z - 1);
+                        float e;
+                        hi[i] = two_sum(hi[i], v[i], e);
+                        lo[i] = two_sum(lo[i], e, q[z]);
+                    }
+                    const float s = __fadd_rn(__fadd_rn(q[0], q[1]), q[2]);
+                    r[0] = __fadd_rn(r[0], s);
+                    if constexpr (cx != 0) r[1] = __fmaf_rn((float)cx, s, r[1]);
+                    if constexpr (cy != 0) r[2] = __fmaf_rn((float)cy, s, r[2]);
+                    r[3] = __fadd_rn(r[3], __fsub_rn(q[2], q[0]));
+                });
             }
         }
-        if (sizeof(R) == 4 && ++held == REDUCE_CELLS) {
-            flush();
-            held = 0;
-        }
     }
-    if (sizeof(R) == 4) flush();
+    if constexpr (sizeof(R) == 4) {
+        double x[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) x[i] = __dadd_rn((double)hi[i], (double)lo[i]);
+        add_sums(acc, moment_sums<double>(x));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] += (double)r[k];
+    }
     block_sum<5>(acc, sh);
     if (threadIdx.x == 0)
 #pragma unroll
