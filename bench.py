@@ -293,7 +293,7 @@ def measured_peak():
 
 # the files that define the step kernel: a traffic figure counts only while they are
 # unchanged since the ncu capture that produced it
-KERNEL_SOURCES = ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_staged.cuh", "lbm_internal.h", "lbm_f32.cu",
+KERNEL_SOURCES = ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_pair.cuh", "lbm_staged.cuh", "lbm_internal.h", "lbm_f32.cu",
                   "lbm_f64.cu", "lbm_f16s.cu", "lbm_bf16.cu")
 
 

@@ -693,7 +693,7 @@ int create_common(lbm_ctx **out, int32_t n, const lbm_grid *grids, const lbm_rel
         off += ceil_div(c->hm[k].scells, 64) * 64;   // keep every member 64-cell aligned
         c->hm[k].doff = doff;
         doff += ceil_div(c->hm[k].cells, 64) * 64;
-        blk += ceil_div(c->hm[k].scells, 128);       // the smallest launch shape
+        blk += ceil_div(c->hm[k].scells, prec == LBM_F64 ? lbm::STEP_SHAPE_F64.threads : 64);   // smallest blocks
         c->grids.push_back(grids[k]);
         c->has_rates.push_back(relax[k].rates != nullptr);
         c->rates.emplace_back();
@@ -702,12 +702,12 @@ int create_common(lbm_ctx **out, int32_t n, const lbm_grid *grids, const lbm_rel
         std::memset(&fz, 0, sizeof fz);
         c->forces.push_back(force ? force[k] : fz);
     }
-    if (blk >= (1ll << 31)) { delete c; return set_err(nullptr, LBM_EINVAL, "grid too large"); }
     if (27 * off >= (1ll << 32)) {
         delete c;
         return set_err(nullptr, LBM_EUNSUPPORTED,
                        "27 x %lld cells exceed the 32-bit population index of the step kernels", (long long)off);
     }
+    if (blk >= (1ll << 31)) { delete c; return set_err(nullptr, LBM_EINVAL, "grid too large"); }
     c->stride = off;
     c->variant_odd = default_variant_odd(prec, wall, off);
     c->dense_total = doff;

@@ -88,8 +88,9 @@ inline void fill_pair_member(PairMember &o, const Member &d) {
 // Programmatic dependent launch.  A step launched with overlap = true may be brought onto the
 // GPU while the step before it drains: it announces its own successor at once, reads its
 // (constant) tables and then waits until every block of the step before it has finished and
-// its writes are visible.  Every step kernel has both calls; without the launch attribute
-// they do nothing.
+// its writes are visible.  The one-cell, pair and adjoint kernels have both calls; without the
+// launch attribute they do nothing.  The pipelined and the staged kernels (shapes 4, 5, 11, 12) have
+// neither: their launchers never set the attribute, with which they would race.
 __device__ __forceinline__ void release_next_step() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void await_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -664,8 +664,8 @@ __device__ __forceinline__ AxisSum<R> axis_sum(R mm, R m0, R mp, R u3, R uh, R u
 
 // One cell (R float or double, any plane) or the cells of planes z and z + 1 (R pf2, no
 // periodic wrap between them) of position r: jterm, wterm their objective and dJ/domega terms.
-// Bound by latency and issue (27 gathers, 9 moments, 27 stores per cell; the 50 MB fields live
-// in L2): pairs share the gather's addresses and halve the arithmetic's issue slots, and the
+// Bound by latency and issue (27 gathers, 9 moments, 27 stores per cell; L2 holds the fields of
+// 50 MB each in part): pairs share the gather's addresses and halve the arithmetic's issue slots, and the
 // axis sums above take 162 operations where psi, psi', psi'' products took 220.  R = 24 pipe,
 // F32: 30 -> 26 us per step (128 threads x 4 blocks, 128 registers, no spills).
 template <int P, int OBJ, class R>
