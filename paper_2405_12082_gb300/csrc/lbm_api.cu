@@ -1329,8 +1329,8 @@ int lbm_autotune(lbm_ctx *c, int32_t steps, int32_t *variant, double *best_us) {
     drop_graph(c);
     // The steps are timed as lbm_step runs them, launches overlapping or as replays of the
     // context's chunk: a step timed apart from its neighbours pays for the launch and the drain
-    // that they hide, which on small pipes is most of it (28 x 28 x 64 pipe, F32: 2.7 us per step
-    // in a row, 4.8 apart), and not the same for every shape.  So each parity's shape is chosen
+    // that they hide, which on small pipes is half of it (28 x 28 x 64 pipe, F32: 3.4 us per step
+    // in a row, 7.3 apart), and not the same for every shape.  So each parity's shape is chosen
     // next to the other's: first the even one beside the present odd one, then the odd one.
     const int32_t chunk = steps >= c->graph_chunk ? c->graph_chunk : 0;
     for (int par = 0; par < 2 && rc == LBM_OK; ++par) {

@@ -12,11 +12,11 @@
 //
 // Why pairs: the step is bound by DRAM (F32) or by the instructions issued per cell at the
 // warps that fit an SM (16-bit).  FFMA2 halves the arithmetic's issue slots (285 -> 145 per
-// cell) and the pair shares the rest: F16S on the R = 48 pipe 686 -> 414 (even) and 903 -> 542
-// (odd) warp instructions per 32 cells, at the same number of cells per SM (16-20 warps of 64
-// cells against 32 of 32).  Measured on the R = 96 pipe, one cell per thread against pairs (us
-// per even / odd step): F32 1143 / 1267 -> 1068 / 1180, F16S 913 / 1040 -> 685 / 866, BF16
-// 908 / 1088 -> 741 / 866.
+// cell, F32 330 -> 165) and the pair shares the rest: F16S on the R = 48 pipe 703 -> 359 (even)
+// and 885 -> 542 (odd) warp instructions per 32 cells, at the same number of cells per SM (14-20
+// warps of 64 or 128 cells against 32 of 32).  Measured on the R = 96 pipe, one cell per thread
+// against pairs (us per even / odd step, timed apart): F32 1143 / 1267 -> 1066 / 1166, F16S
+// 913 / 1040 -> 639 / 861, BF16 908 / 1088 -> 630 / 867.
 #pragma once
 
 #include "lbm_internal.h"
@@ -195,8 +195,8 @@ __device__ __forceinline__ void even_pair(const A &a, const D &d, int m, uint32_
 
 // Two pairs per thread in the 16-bit formats with half-way walls (even_pairs): one 8-byte access
 // loads a population of four cells, so the second pair's values wait in 27 registers while the
-// first is collided, and the addresses serve both (R = 96 pipe: BF16 750 -> 662 us, F16S 687 ->
-// 681).  In F32 the second pair would take 54 registers, and with Bouzidi walls the outputs of a
+// first is collided, and the addresses serve both (R = 96 pipe, when it was made: BF16 750 -> 662
+// us, F16S 687 -> 681; now 630 and 639).  In F32 the second pair would take 54 registers, and with Bouzidi walls the outputs of a
 // pair are held as well (860 -> 1,002 us in F16S): one pair there.
 template <int P, int WALL, int EXTRA, int BS, int MINB, class A>
 __global__ void __launch_bounds__(BS, MINB) k_even2(const __grid_constant__ A a) {
